@@ -672,30 +672,55 @@ __global__ void __launch_bounds__(kUpdThreads) k_update_batch(const UpdateArgs* 
                  __ldg(thread_start + lo + 1) - __ldg(thread_start + lo));
 }
 
-// Warm start: one thread per control dimension walks the horizon forward (in
-// place is safe: row t reads row t+k >= t); the last row repeats.
-__device__ __forceinline__ void shift_body(double* mu, double* sigma, float* mu_f, float* sigma_f,
-                                           int H, int n, int k, int i) {
-  for (int t = 0; t < H; ++t) {
-    const int src = t + k < H ? t + k : H - 1;
-    mu[t * n + i] = mu[src * n + i];
-    sigma[t * n + i] = sigma[src * n + i];
-    mu_f[t * n + i] = (float)mu[t * n + i];
-    sigma_f[t * n + i] = (float)sigma[t * n + i];
+// Warm start of one instance by one block: element e = t n + i takes the value
+// k steps later, the last row's past the end.  In place: a block pass first
+// reads its elements' sources (none lies before the pass, and the last row,
+// the only source that is also written, keeps its values), then writes them.
+// Each thread moves kShiftBatch elements per pass, their loads in flight
+// together.  Bound by the latency of the passes' loads.  One thread per
+// control dimension walking the horizon, as before, waited for H dependent
+// loads: a serving cycle of 48 robots spent 93 us here (ncu, cold), now 5.
+constexpr int kShiftThreads = 256;
+constexpr int kShiftBatch = 4;
+
+__device__ __forceinline__ void shift_body(double* mu, double* sigma, float* mu_f, float* sigma_f, int H,
+                                           int n, int k) {
+  const long long Hn = (long long)H * n, off = (long long)k * n;
+  for (long long e0 = threadIdx.x; e0 - threadIdx.x < Hn; e0 += kShiftBatch * kShiftThreads) {
+    double m[kShiftBatch], s[kShiftBatch];
+#pragma unroll
+    for (int j = 0; j < kShiftBatch; ++j) {
+      const long long e = e0 + j * kShiftThreads;
+      if (e < Hn) {
+        const long long src = e + off < Hn ? e + off : Hn - n + e % n;
+        m[j] = mu[src];
+        s[j] = sigma[src];
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < kShiftBatch; ++j) {
+      const long long e = e0 + j * kShiftThreads;
+      if (e < Hn) {
+        mu[e] = m[j];
+        sigma[e] = s[j];
+        mu_f[e] = (float)m[j];
+        sigma_f[e] = (float)s[j];
+      }
+    }
+    __syncthreads();
   }
 }
 
-__global__ void k_shift(double* mu, double* sigma, float* mu_f, float* sigma_f, int H, int n,
-                        int k) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) shift_body(mu, sigma, mu_f, sigma_f, H, n, k, i);
+__global__ void __launch_bounds__(kShiftThreads) k_shift(double* mu, double* sigma, float* mu_f, float* sigma_f,
+                                                         int H, int n, int k) {
+  shift_body(mu, sigma, mu_f, sigma_f, H, n, k);
 }
 
 // one block per instance of a batch
-__global__ void k_shift_batch(const UpdateArgs* __restrict__ args, int k) {
+__global__ void __launch_bounds__(kShiftThreads) k_shift_batch(const UpdateArgs* __restrict__ args, int k) {
   const UpdateArgs& a = args[blockIdx.x];
-  for (int i = threadIdx.x; i < a.n; i += blockDim.x)
-    shift_body(a.mu, a.sigma, a.mu_f, a.sigma_f, a.H, a.n, k, i);
+  shift_body(a.mu, a.sigma, a.mu_f, a.sigma_f, a.H, a.n, k);
 }
 
 }  // namespace
@@ -814,13 +839,13 @@ cudaError_t launch_update(const UpdateArgs& a, cudaStream_t s) {
 
 cudaError_t launch_shift_batch(const UpdateArgs* d_args, int count, int k, cudaStream_t s) {
   if (count <= 0 || k <= 0) return cudaSuccess;
-  k_shift_batch<<<count, 32, 0, s>>>(d_args, k);
+  k_shift_batch<<<count, kShiftThreads, 0, s>>>(d_args, k);
   return cudaGetLastError();
 }
 
 cudaError_t launch_shift(double* mu, double* sigma, float* mu_f, float* sigma_f, int H, int n, int k,
                          cudaStream_t s) {
-  k_shift<<<(n + 63) / 64, 64, 0, s>>>(mu, sigma, mu_f, sigma_f, H, n, k);
+  k_shift<<<1, kShiftThreads, 0, s>>>(mu, sigma, mu_f, sigma_f, H, n, k);
   return cudaGetLastError();
 }
 

@@ -142,6 +142,7 @@ def fp32_peak(sm_mhz: float, sms: int) -> tuple[float, str]:
 
 KERNEL_HEADERS = ("paper_2505_01059_gb300/csrc/rollout_common.cuh",
                   "paper_2505_01059_gb300/csrc/rollout_kernels.cuh",
+                  "paper_2505_01059_gb300/csrc/rollout_pm.cuh",
                   "paper_2505_01059_gb300/csrc/mtp_device.cuh", "include/mtp.h")
 KERNEL_FILE = {"pointmass": "rollout_pm.cu", "chain": "rollout_chain.cu", "legged": "legged.cu"}
 BATCH_KERNEL_FILE = {"pointmass": "rollout_pm_batch.cu", "chain": "rollout_chain_batch.cu",

@@ -334,15 +334,14 @@ mtp_status mtp_batch_plan_step(mtp_batch* b, const float* d_x0, int32_t iters, f
                                void* stream);
 
 /* Picks the rollout tile of each (dynamics, dimension) group by timing its
- * rollout launch (best of three) for every choice: candidates per block (32,
- * 64 or 128) times the horizon chunk of the staged control loads (0: direct
- * loads; 4 or 8 steps of every candidate's controls copied at once into
+ * rollout launch (best of three) for every choice: threads per block (32, 64
+ * or 128) and, for chains, the horizon chunk of the staged control loads (0:
+ * direct loads; 4 steps of every candidate's controls copied at once into
  * shared memory by bulk copies, when every member's rows allow it: 16-byte
- * aligned, H * n a multiple of 4, one model per candidate), and for point
- * masses also two candidates per thread (64 per warp, direct loads).  The
- * legged group keeps its fixed tile.  Writes (dynamics, dimension, block,
- * chunk, candidates per thread) to tiles_out (5 * groups entries, may be
- * NULL) and the number of groups to n_groups.  Then it picks the rollout
+ * aligned, H * n a multiple of 4, one model per candidate).  The legged group
+ * keeps its fixed tile.  Writes (dynamics, dimension, block, chunk, candidates
+ * per thread: 1) to tiles_out (5 * groups entries, may be NULL) and the number
+ * of groups to n_groups.  Then it picks the rollout
  * mode (mtp_batch_set_rollout_mode) by timing whole iterations in each mode,
  * each captured as the CUDA graph that mtp_batch_plan_step replays (best of
  * three replays after one untimed one), with every instance's planner state
@@ -362,10 +361,9 @@ mtp_status mtp_batch_autotune(mtp_batch* b, int32_t* tiles_out, int32_t* n_group
  *   one persistent launch, after all instances' candidates are made: each
  *   warp takes warp tiles of 32 candidates of one instance from a device
  *   counter, group by group (the longest group first, within a group the
- *   longest expected rollout first: H times the group's time per step),
- *   with their controls staged through shared memory 4 steps at a
- *   time where the instance's rows allow it (_STAGED) or loaded directly
- *   (_DIRECT).  Legged robots and longer chains keep their own launches
+ *   longest expected rollout first: H times the group's time per step).
+ *   A chain's controls are staged through shared memory 4 steps at a time
+ *   where the instance's rows allow it (_STAGED) or loaded directly (_DIRECT).  Legged robots and longer chains keep their own launches
  *   beside it.  The launch is counted as one kernel by mtp_batch_launches.
  * MTP_BATCH_ROLLOUT_PERSISTENT_SPLIT: the same with staged tiles, in two
  *   persistent launches split at a group boundary near 65 % of the expected

@@ -28,9 +28,7 @@ struct BatchGroup {
   int total_rows = 0;
   int block = 128;
   int chunk = 0;              // horizon chunk of staged control loads (0: direct loads)
-  int samples = 1;            // candidates per thread (point masses: 1 or 2, direct loads)
   bool stageable = false;     // every member's rows can be staged (see can_stage)
-  bool pairable = false;      // point masses with one model per candidate: 2 per thread allowed
   // this group's share of the generation, selection and update launches
   int z_blocks = 0, cand_blocks = 0, local_blocks = 0, upd_threads = 0;
   // members whose graph rows are contracted on the tensor cores (BF16 basis):
@@ -149,9 +147,8 @@ struct mtp_batch {
   BatchTables t;
   int count = 0;
   std::vector<BatchGroup> groups;
-  // (dyn, n) -> rollout tile chosen by the autotuner: (candidates per block, horizon chunk,
-  // candidates per thread)
-  std::map<std::pair<int, int>, std::array<int, 3>> tuned;
+  // (dyn, n) -> rollout tile chosen by the autotuner: (threads per block, horizon chunk)
+  std::map<std::pair<int, int>, std::array<int, 2>> tuned;
   // (dyn, n) -> the autotuner's rollout time of the group (ms) per rollout step
   std::map<std::pair<int, int>, double> tuned_ms_per_step;
   // groups in launch order: longest expected rollout first
@@ -177,7 +174,7 @@ struct mtp_batch {
   cudaStream_t persist_stream[2] = {nullptr, nullptr};
   cudaEvent_t persist_ev2 = nullptr;
   cudaStream_t group_stream_hi[kMaxGroups] = {};  // high priority: the first launch's generation
-  size_t p_warp_bytes = 0;      // staged tiles' shared memory per warp (0: none stageable)
+  size_t p_warp_bytes[2] = {0, 0};  // shared memory per warp: staged mode, direct mode
   int p_blocks[2] = {0, 0};     // resident CTAs per SM: staged mode, direct mode
   cudaEvent_t persist_ev = nullptr;
   double mode_ms[4] = {0, 0, 0, 0};  // the autotuner's iteration time per mode (0: not timed)
@@ -305,7 +302,6 @@ cudaError_t fill_batch(mtp_batch* b, mtp_handle* const* handles, int count, cuda
       auto it = b->tuned.find({dyn, n});
       g.block = it != b->tuned.end() ? it->second[0] : 128;
       g.chunk = it != b->tuned.end() ? it->second[1] : kDefaultChunk;
-      g.samples = it != b->tuned.end() ? it->second[2] : 1;
       b->groups.push_back(g);
     }
     ++b->groups.back().count;
@@ -410,21 +406,13 @@ cudaError_t fill_batch(mtp_batch* b, mtp_handle* const* handles, int count, cuda
       if (g.dyn == MTP_DYN_POINTMASS) hv.d_pm[m] = pointmass_model(h->pr);
       else if (g.dyn == MTP_DYN_LEGGED) hv.d_lm[m] = legged_model(h->pr);
       else hv.d_cm[m] = chain_model(h->pr);
-      // whole warps per instance; point masses whole pairs of warps (two
-      // candidates per thread take rows 32 apart)
-      const int pad = g.dyn == MTP_DYN_POINTMASS ? 64 : 32;
-      row[j + 1] = row[j] + ((h->dm.B + pad - 1) / pad) * pad;
+      row[j + 1] = row[j] + ((h->dm.B + 31) / 32) * 32;  // whole warps per instance
     }
     g.total_rows = row[g.count];
-    g.stageable = g.dyn != MTP_DYN_LEGGED;
+    g.stageable = g.dyn == MTP_DYN_CHAIN;
     for (int j = 0; j < g.count; ++j)
       g.stageable = g.stageable && can_stage(hv.d_ra[g.first + j], group_key_n(handles[order[g.first + j]]));
     if (!g.stageable) g.chunk = 0;
-    g.pairable = g.dyn == MTP_DYN_POINTMASS;
-    for (int j = 0; j < g.count; ++j)
-      g.pairable = g.pairable && hv.d_ra[g.first + j].dr_mode != MTP_DR_SHARED;
-    if (!g.pairable) g.samples = 1;
-    if (g.samples == 2) g.chunk = 0;
     rs += g.count + 1;
   }
   set_launch_order(b, [&](const BatchGroup& g) {
@@ -444,7 +432,8 @@ cudaError_t fill_batch(mtp_batch* b, mtp_handle* const* handles, int count, cuda
       int pos, code, model, warps;
     };
     std::vector<Entry> ent;
-    int max_pm = 0, max_links = 0;
+    size_t pm_floats = 0;
+    int max_links = 0;
     for (size_t gi = 0; gi < b->groups.size(); ++gi) {
       const BatchGroup& g = b->groups[gi];
       const bool cov = (g.dyn == MTP_DYN_POINTMASS && g.n <= kPersistMaxAxes) ||
@@ -459,8 +448,8 @@ cudaError_t fill_batch(mtp_batch* b, mtp_handle* const* handles, int count, cuda
         const int pos = g.first + j;
         const mtp_handle* h = handles[order[pos]];
         const bool stage = can_stage(hv.d_ra[pos], g.n);
-        if (stage) (g.dyn == MTP_DYN_POINTMASS ? max_pm : max_links) = std::max(
-                       g.dyn == MTP_DYN_POINTMASS ? max_pm : max_links, g.n);
+        if (g.dyn == MTP_DYN_POINTMASS) pm_floats = std::max(pm_floats, persist_pm_floats(g.n));
+        else if (stage) max_links = std::max(max_links, g.n);
         ent.push_back({per_step * h->dm.H, pos, g.dyn | (g.n << 8) | (stage ? 1 << 16 : 0),
                        g.model_first + j, (h->dm.B + 31) / 32});
       }
@@ -518,9 +507,9 @@ cudaError_t fill_batch(mtp_batch* b, mtp_handle* const* handles, int count, cuda
     }
     b->p_count = (int)ent.size();
     b->p_total_warps = w;
-    b->p_warp_bytes = persist_warp_bytes(max_pm, max_links);
-    b->p_blocks[0] = persist_blocks_per_sm(b->p_warp_bytes);
-    b->p_blocks[1] = persist_blocks_per_sm(0);
+    b->p_warp_bytes[0] = persist_warp_bytes(pm_floats, max_links);
+    b->p_warp_bytes[1] = persist_warp_bytes(pm_floats, 0);
+    for (int k = 0; k < 2; ++k) b->p_blocks[k] = persist_blocks_per_sm(b->p_warp_bytes[k]);
     if (b->p_count > 0 && (b->p_blocks[0] < 1 || b->p_blocks[1] < 1)) return cudaErrorInvalidConfiguration;
   }
   // packing of x0 and u*, in the caller's order
@@ -556,17 +545,13 @@ cudaError_t fill_batch(mtp_batch* b, mtp_handle* const* handles, int count, cuda
   return cudaSuccess;
 }
 
-cudaError_t launch_group(const mtp_batch* b, const BatchGroup& g, int block, int chunk, int samples,
-                         cudaStream_t s) {
+cudaError_t launch_group(const mtp_batch* b, const BatchGroup& g, int block, int chunk, cudaStream_t s) {
   const BatchTables& t = b->t;
   const RolloutArgs* ra = t.d_ra + g.first;
   const int* rs = t.d_row_start + g.rows_first;
   if (!g.stageable) chunk = 0;
-  if (!g.pairable) samples = 1;
-  if (samples == 2) chunk = 0;
   if (g.dyn == MTP_DYN_POINTMASS)
-    return launch_rollout_pointmass_batch(ra, t.d_pm + g.model_first, rs, g.count, g.total_rows, g.n,
-                                          block, chunk, samples, s);
+    return launch_rollout_pointmass_batch(ra, t.d_pm + g.model_first, rs, g.count, g.total_rows, g.n, block, s);
   if (g.dyn == MTP_DYN_LEGGED)  // fixed 64-thread blocks (shared-memory staging)
     return launch_rollout_legged_batch(ra, t.d_lm + g.model_first, rs, g.count, g.total_rows, g.n, s);
   return launch_rollout_chain_batch(ra, t.d_cm + g.model_first, rs, g.count, g.total_rows, g.n, block,
@@ -594,7 +579,8 @@ PersistArgs persist_args(const mtp_batch* b, bool staged, int part = 0) {
   p.count = b->p_count;
   p.total_warps = b->p_total_warps;
   p.w_base = 0;
-  p.warp_bytes = staged ? b->p_warp_bytes : 0;
+  p.warp_bytes = b->p_warp_bytes[staged ? 0 : 1];
+  p.staged = staged ? 1 : 0;
   if (part == 1) {
     p.count = b->p_split;
     p.total_warps = b->p_split_warps;
@@ -642,7 +628,7 @@ cudaError_t enqueue_batch_iteration_persistent(mtp_batch* b, cudaStream_t s, boo
       return e;
     if ((e = launch_local_batch(t.d_cand + f, t.d_local_start + f, g.count, g.local_blocks, gs))) return e;
     if (!b->covered[gi]) {
-      if ((e = launch_group(b, g, g.block, g.chunk, g.samples, gs))) return e;
+      if ((e = launch_group(b, g, g.block, g.chunk, gs))) return e;
       if ((e = launch_select_batch(t.d_sel + f, g.count, g.sel_smem, gs))) return e;
       if ((e = launch_update_batch(t.d_upd + f, t.d_warp_start + f, g.count, g.upd_threads, gs))) return e;
     }
@@ -706,7 +692,7 @@ cudaError_t enqueue_batch_iteration(mtp_batch* b, cudaStream_t s) {
                                      g.tc_tiles, gs)))
       return e;
     if ((e = launch_local_batch(t.d_cand + f, t.d_local_start + f, g.count, g.local_blocks, gs))) return e;
-    if ((e = launch_group(b, g, g.block, g.chunk, g.samples, gs))) return e;
+    if ((e = launch_group(b, g, g.block, g.chunk, gs))) return e;
     if ((e = launch_select_batch(t.d_sel + f, g.count, g.sel_smem, gs))) return e;
     if ((e = launch_update_batch(t.d_upd + f, t.d_warp_start + f, g.count, g.upd_threads, gs))) return e;
     if ((e = cudaEventRecord(b->group_done[gi], gs))) return e;
@@ -970,22 +956,20 @@ mtp_status mtp_batch_autotune(mtp_batch* b, int32_t* tiles_out, int32_t* n_group
   DeviceGuard guard(b->device);
   (void)stream;
   cudaEventSynchronize(b->t.copied);  // the tables may have been filled on another stream
-  // rollout tiles: candidates per block (the kernels are bounded at 128
-  // threads) x horizon chunk of the staged control loads (0: direct loads)
+  // rollout tiles: threads per block (the kernels are bounded at 128) x, for
+  // chains, the horizon chunk of the staged control loads (0: direct loads)
   const int blocks[3] = {32, 64, 128};
-  const int chunks[3] = {0, 4, 8};  // chains stage 4 steps at a time (8 is not tried)
+  const int chunks[2] = {0, 4};
   cudaEvent_t t0, t1;
   cudaEventCreate(&t0);
   cudaEventCreate(&t1);
   cudaError_t e = cudaSuccess;
-  // tiles: (candidates per block, horizon chunk, candidates per thread)
   struct Tile {
-    int block, chunk, samples;
+    int block, chunk;
   };
   std::vector<Tile> tiles;
   for (int chunk : chunks)
-    for (int block : blocks) tiles.push_back({block, chunk, 1});
-  for (int block : blocks) tiles.push_back({block, 0, 2});
+    for (int block : blocks) tiles.push_back({block, chunk});
   auto group_steps = [&](const BatchGroup& g) {
     long long steps = 0;
     for (int j = 0; j < g.count; ++j) steps += (long long)b->hs_sorted[g.first + j]->dm.B * b->hs_sorted[g.first + j]->dm.H;
@@ -993,17 +977,15 @@ mtp_status mtp_batch_autotune(mtp_batch* b, int32_t* tiles_out, int32_t* n_group
   };
   for (auto& g : b->groups) {
     float best = 1e30f;
-    Tile best_tile{g.block, g.chunk, g.samples};
+    Tile best_tile{g.block, g.chunk};
     for (const Tile& tl : tiles) {
       // the legged rollout has one fixed tile: timed once, for the launch order
-      if (g.dyn == MTP_DYN_LEGGED && (tl.block != blocks[0] || tl.chunk || tl.samples != 1)) continue;
+      if (g.dyn == MTP_DYN_LEGGED && (tl.block != blocks[0] || tl.chunk)) continue;
       if (tl.chunk && !g.stageable) continue;
-      if (tl.chunk == 8 && g.dyn == MTP_DYN_CHAIN) continue;
-      if (tl.samples == 2 && !g.pairable) continue;
       float ms_min = 1e30f;
       for (int rep = 0; rep < 3 && e == cudaSuccess; ++rep) {
         cudaEventRecord(t0, b->cap_stream);
-        e = launch_group(b, g, tl.block, tl.chunk, tl.samples, b->cap_stream);
+        e = launch_group(b, g, tl.block, tl.chunk, b->cap_stream);
         cudaEventRecord(t1, b->cap_stream);
         cudaEventSynchronize(t1);
         float ms = 0.f;
@@ -1020,8 +1002,7 @@ mtp_status mtp_batch_autotune(mtp_batch* b, int32_t* tiles_out, int32_t* n_group
     if (g.dyn == MTP_DYN_LEGGED) continue;
     g.block = best_tile.block;
     g.chunk = best_tile.chunk;
-    g.samples = best_tile.samples;
-    b->tuned[{g.dyn, g.n}] = {g.block, g.chunk, g.samples};
+    b->tuned[{g.dyn, g.n}] = {g.block, g.chunk};
   }
   set_launch_order(b, group_steps);
   cudaEventDestroy(t0);
@@ -1044,7 +1025,7 @@ mtp_status mtp_batch_autotune(mtp_batch* b, int32_t* tiles_out, int32_t* n_group
       tiles_out[5 * i + 1] = b->groups[i].n;
       tiles_out[5 * i + 2] = b->groups[i].block;
       tiles_out[5 * i + 3] = b->groups[i].chunk;
-      tiles_out[5 * i + 4] = b->groups[i].samples;
+      tiles_out[5 * i + 4] = 1;  // one candidate per thread
     }
   return MTP_OK;
 }
@@ -1139,7 +1120,7 @@ mtp_status mtp_batch_rollout_times(mtp_batch* b, int32_t reps, double* ms_out, i
     double sum = 0.0;
     for (int rep = 0; rep < reps && e == cudaSuccess; ++rep) {
       if ((e = cudaEventRecord(t0, s))) break;
-      if ((e = launch_group(b, g, g.block, g.chunk, g.samples, s))) break;
+      if ((e = launch_group(b, g, g.block, g.chunk, s))) break;
       if ((e = cudaEventRecord(t1, s))) break;
       if ((e = cudaEventSynchronize(t1))) break;
       float ms = 0.f;
@@ -1162,7 +1143,7 @@ mtp_status mtp_batch_rollout_times(mtp_batch* b, int32_t reps, double* ms_out, i
       o[4] = (int32_t)rows;
       o[5] = (int32_t)std::min<long long>(steps, 0x7fffffff);
       o[6] = g.stageable ? g.chunk : 0;
-      o[7] = g.pairable ? g.samples : 1;
+      o[7] = 1;
     }
   }
   cudaEventDestroy(t0);

@@ -414,7 +414,7 @@ cudaError_t launch_selection(const mtp_handle* h, const SelectArgs& a, cudaStrea
 
 cudaError_t launch_rollout(const mtp_handle* h, const RolloutArgs& a, cudaStream_t s) {
   const mtp_problem& p = h->pr;
-  if (p.dyn == MTP_DYN_POINTMASS) return launch_rollout_pointmass(a, pointmass_model(p), h->rollout_chunk, s);
+  if (p.dyn == MTP_DYN_POINTMASS) return launch_rollout_pointmass(a, pointmass_model(p), s);
   if (p.dyn == MTP_DYN_LEGGED) return launch_rollout_legged(a, legged_model(p), p.n_links, s);
   return launch_rollout_chain(a, chain_model(p), p.n_links, h->rollout_chunk, s);
 }
@@ -472,7 +472,10 @@ cudaError_t enqueue_iteration(mtp_handle* h, cudaStream_t s, int work, Gen gen, 
   }
   if (e != cudaSuccess) return e;
   if (ev) stage_event(ev[1], s, captured);
-  if (h->pipeline) {
+  // the next iteration's graph rows and draws on the side stream: beside the
+  // rollout, on the SMs it leaves idle, or after a point-mass rollout (a few
+  // microseconds on every SM), beside the selection's one block
+  auto prepare_next = [&]() -> cudaError_t {
     if ((e = cudaEventRecord(h->ev_fork, s)) != cudaSuccess) return e;
     if ((e = cudaStreamWaitEvent(h->side, h->ev_fork, 0)) != cudaSuccess) return e;
     if (ev) stage_event(ev[5], h->side, captured);
@@ -486,10 +489,14 @@ cudaError_t enqueue_iteration(mtp_handle* h, cudaStream_t s, int work, Gen gen, 
     if ((e = launch_prepare(nx, h->prep_grid, h->prep_smem, h->side)) != cudaSuccess) return e;
     if (ev) stage_event(ev[6], h->side, captured);
     if ((e = cudaEventRecord(h->ev_join, h->side)) != cudaSuccess) return e;
-  }
+    return cudaSuccess;
+  };
+  const bool beside_rollout = h->pr.dyn != MTP_DYN_POINTMASS;
+  if (h->pipeline && beside_rollout && (e = prepare_next()) != cudaSuccess) return e;
   RolloutArgs r = rollout_args(h, 0, h->iter_dev, h->x0, U, 0, dm.B, h->cost);
   if ((e = launch_rollout(h, r, s)) != cudaSuccess) return e;
   if (ev) stage_event(ev[2], s, captured);
+  if (h->pipeline && !beside_rollout && (e = prepare_next()) != cudaSuccess) return e;
   SelectArgs sa{h->cost, U, dm.B, dm.E, dm.H, dm.n, 1.0 / h->pr.lambda, h->pr.update_rule,
                 h->elite, h->weight, h->ustar, nullptr, ustar_out, h->entropy, h->sel_pairs, 0};
   if ((e = launch_selection(h, sa, s)) != cudaSuccess) return e;
@@ -628,7 +635,8 @@ cudaError_t pipeline_plan(const mtp_problem& p, const Dims& dm, int paths_per_bl
   *prep_spb = std::max(probe.paths_per_block, paths_per_block);
   *on = true;
   *local = draws;
-  *grid = free_sms;
+  // a point mass's preparation runs beside the selection, which takes one SM
+  *grid = p.dyn == MTP_DYN_POINTMASS ? sms - 1 : free_sms;
   return cudaSuccess;
 }
 

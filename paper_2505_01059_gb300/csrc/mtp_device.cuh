@@ -248,8 +248,7 @@ cudaError_t init_rollout_pm_attributes();
 cudaError_t init_rollout_chain_attributes();
 cudaError_t init_rollout_pm_batch_attributes();
 cudaError_t init_rollout_chain_batch_attributes();
-cudaError_t launch_rollout_pointmass(const RolloutArgs& a, const PointMassModel& m, int chunk,
-                                     cudaStream_t s);
+cudaError_t launch_rollout_pointmass(const RolloutArgs& a, const PointMassModel& m, cudaStream_t s);
 cudaError_t launch_rollout_chain(const RolloutArgs& a, const ChainModel& m, int links, int chunk,
                                  cudaStream_t s);
 cudaError_t launch_rollout_legged(const RolloutArgs& a, const LeggedModel& m, int links,
@@ -278,10 +277,14 @@ struct PersistArgs {
   unsigned* head;     // the tile counter, zeroed by the launch
   int count, total_warps;
   int w_base;         // wstart[0]: the first tile of these entries in the batch's numbering
-  size_t warp_bytes;  // shared memory per warp: two mbarriers and two staging buffers (0: no staging)
+  size_t warp_bytes;  // shared memory per warp: two mbarriers and the largest tile
+  int staged;         // chain tiles stage their controls where their rows allow it (else direct loads)
 };
-// Shared memory per warp for staged tiles of at most these widths (0: none).
-size_t persist_warp_bytes(int max_pm_axes_staged, int max_links_staged);
+// Shared memory per warp: a point mass's tile of `axes` axes, in floats; and
+// all of a warp's, for point-mass tiles of at most pm_floats and staged chain
+// tiles of at most max_links_staged links (0: none staged).
+size_t persist_pm_floats(int axes);
+size_t persist_warp_bytes(size_t pm_floats, int max_links_staged);
 // Resident 128-thread CTAs per SM of the persistent launch with that much
 // shared memory per warp (0 on error); also sets the launch's shared-memory
 // attribute.
@@ -326,8 +329,7 @@ cudaError_t launch_candidates_batch(const CandArgs* d_args, const int* d_block_s
                                     int total_blocks, size_t smem, cudaStream_t s);
 cudaError_t launch_rollout_pointmass_batch(const RolloutArgs* d_ra, const PointMassModel* d_pm,
                                            const int* d_row_start, int count, int total_rows,
-                                           int k, int block, int chunk, int samples,
-                                           cudaStream_t s);
+                                           int k, int block, cudaStream_t s);
 cudaError_t launch_rollout_chain_batch(const RolloutArgs* d_ra, const ChainModel* d_cm,
                                        const int* d_row_start, int count, int total_rows,
                                        int links, int block, int chunk, cudaStream_t s);

@@ -8,7 +8,7 @@
 namespace mtp {
 namespace {
 
-// Control steps requested ahead of use by the point-mass and chain rollouts.
+// Control steps requested ahead of use by the chain rollouts.
 // Measured on GB300 (depths 1 / 2 / 3 / 4): a lone instance, which has one
 // warp per SM sub-partition at most, is fastest at 2 (7-link arm 118 / 105 /
 // 105 / 109 us per step); a batch, where registers set how many warps are

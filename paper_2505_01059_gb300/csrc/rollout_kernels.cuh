@@ -1,16 +1,15 @@
 // rollout_kernels.cuh -- Alg. 2 batch rollout fused with the cost reduction
-// (Eq. 2) for the k-D point mass and the planar serial chain: the device
-// bodies and kernels, instantiated by rollout_pm.cu and rollout_chain.cu.
+// (Eq. 2) for the planar serial chain: the device body and kernels,
+// instantiated by rollout_chain.cu, rollout_chain_batch.cu and
+// rollout_persist.cu.
 //
 // One thread per candidate keeps the whole state in registers for all H
 // steps and accumulates c(x_t, u_t) with compensated FP32 sums; only the
 // final cost leaves the SM.  The loop bodies are fully unrolled over the
-// compile-time dimension (point-mass axes, chain links), so the per-step
-// linear algebra lives in registers.  The controls reach a thread either by
-// direct loads a few steps ahead (T = 0) or staged through shared memory a
-// horizon chunk of T steps at a time by bulk copies (T = 4, 8; see
-// StagedRows): the chunk length is the rollout tile's horizon chunk, picked
-// per launch shape by the batch autotuner.
+// compile-time link count, so the per-step linear algebra lives in registers.
+// The controls reach a thread either by direct loads a few steps ahead (T = 0)
+// or staged through shared memory a horizon chunk of T = 4 steps at a time by
+// bulk copies (see StagedRows), picked per launch shape by the batch autotuner.
 //
 // Planar chain: the dynamics are evaluated in absolute link angles phi_j
 // (phi_j = q_1 + ... + q_j).  For uniform thin rods the Lagrangian gives the
@@ -65,173 +64,8 @@ __device__ __forceinline__ void report_stage_timeout(const RolloutArgs& a) {
 }
 
 // ---------------------------------------------------------------------------
-// k-D point mass (double integrator), control = acceleration x gain.
-// ---------------------------------------------------------------------------
-// ALL: every obstacle slot is evaluated, with no branch (the slots past
-// n_obs have radius 0 and add exactly +0): one basic block, so the obstacles'
-// SFU latencies overlap, for a lone latency-bound instance (measured on the
-// C1 point mass: rollout 26.0 -> 20.5 us).  Otherwise the slots past n_obs
-// are skipped, which saves their instructions where many instances keep the
-// GPU busy (the batch of 256: 3.84 -> 3.72 ms).  The sums are the same bits.
-template <int K, bool ALL>
-__device__ __forceinline__ float pm_state_cost(const PointMassModel& pm, const float (&p)[K]) {
-  float dist2 = 0.f;
-#pragma unroll
-  for (int k = 0; k < K; ++k) {
-    const float e = p[k] - pm.target[k];
-    dist2 = fmaf(e, e, dist2);
-  }
-  // unrolled to the maximum obstacle count so every model index is a
-  // constant (a run-time index into the kernel parameters goes through the
-  // constant cache's slow indexed path)
-  float pen = 0.f;
-#pragma unroll
-  for (int o = 0; o < MTP_MAX_OBSTACLES; ++o) {
-    if (ALL || o < pm.n_obs) {
-      float d2 = 0.f;
-#pragma unroll
-      for (int k = 0; k < K; ++k) {
-        const float e = p[k] - pm.obs_c[o][k];
-        d2 = fmaf(e, e, d2);
-      }
-      // distance as d2 * rsqrt(d2): one SFU operation and a multiply instead
-      // of the correctly rounded square root's fix-up sequence (relative
-      // error ~1e-7, far inside the cost tolerance)
-      const float dist = d2 > 0.f ? d2 * rsqrtf(d2) : 0.f;
-      const float depth = pm.obs_r[o] - dist;
-      pen += depth > 0.f ? depth : 0.f;
-    }
-  }
-  return fmaf(pm.w_target, dist2, pm.w_obs * pen);
-}
-
-// The K controls of step t drive v += dt g u, p += dt v (g: the per-model
-// control gains of the domain randomisation); the stage cost is taken
-// before the step and the terminal cost on the final state.
-template <int K, int PF, bool ALL, int T>
-__device__ __forceinline__ bool rollout_pm_body(const RolloutArgs& a, const PointMassModel& pm,
-                                                int r, bool live, StagedRows<K, T>* st) {
-  const int b = a.row0 + r;
-  const uint32_t iter = a.d_iter ? *a.d_iter : a.iter;
-  const float* Ub = a.U + (size_t)r * a.H * K;
-  const int models = (a.dr_mode == MTP_DR_SHARED) ? a.R : 1;
-  const float dt = a.dt;
-  float total = 0.f;
-  bool ok = true;
-  for (int mdl = 0; mdl < models && ok; ++mdl) {
-    const uint32_t unit = (a.dr_mode == MTP_DR_SHARED) ? (uint32_t)mdl : (uint32_t)b;
-    float gain[K], p[K], v[K];
-    dr_scales<K>(a, iter, unit, gain);
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-      gain[k] *= dt;
-      p[k] = a.x0[k];
-      v[k] = a.x0[K + k];
-    }
-    if (a.X) {
-#pragma unroll
-      for (int k = 0; k < K; ++k) {
-        a.X[k] = p[k];
-        a.X[K + k] = v[k];
-      }
-    }
-    KahanSum J;
-    ok = for_each_step<K, PF, T>(Ub, a.H, st, [&](int t, const float (&u)[K]) {
-      float uu = 0.f;
-#pragma unroll
-      for (int k = 0; k < K; ++k) uu = fmaf(u[k], u[k], uu);
-      J.add(fmaf(pm.w_ctrl, uu, pm_state_cost<K, ALL>(pm, p)), a.kahan);
-#pragma unroll
-      for (int k = 0; k < K; ++k) {
-        v[k] = fmaf(gain[k], u[k], v[k]);
-        p[k] = fmaf(dt, v[k], p[k]);
-      }
-      if (a.X) {
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-          a.X[(size_t)(t + 1) * 2 * K + k] = p[k];
-          a.X[(size_t)(t + 1) * 2 * K + K + k] = v[k];
-        }
-      }
-    });
-    J.add(pm.w_term * pm_state_cost<K, ALL>(pm, p), a.kahan);
-    total += J.s;
-  }
-  if (!live) return ok;
-  float c = total / (float)models;
-  if (!isfinite(c) || !ok) c = __int_as_float(0x7f800000);
-  if (!ok) report_stage_timeout(a);
-  a.cost[r] = c;
-  return ok;
-}
-
-// ---------------------------------------------------------------------------
 // Planar serial chain under joint torques.
 // ---------------------------------------------------------------------------
-// Two candidates per thread (rows r[0] and r[1] of one instance, 32 rows
-// apart), direct loads one step ahead, one model: the two chains of
-// dependent instructions interleave, which the point-mass step needs (its
-// warps otherwise stall on fixed-latency dependencies most of the time).
-// Same arithmetic per candidate as rollout_pm_body, so the same bits.  A
-// candidate without a row (live false) reads the instance's first row and
-// writes nothing.  One model per candidate (no shared-model averaging).
-template <int K>
-__device__ __forceinline__ void rollout_pm_pair(const RolloutArgs& a, const PointMassModel& pm,
-                                                const int (&r)[2], const bool (&live)[2]) {
-  constexpr int S = 2;
-  const uint32_t iter = a.d_iter ? *a.d_iter : a.iter;
-  const float dt = a.dt;
-  const int H = a.H;
-  const float* Ub[S];
-  float gain[S][K], p[S][K], v[S][K];
-  KahanSum J[S];
-#pragma unroll
-  for (int c = 0; c < S; ++c) {
-    Ub[c] = a.U + (size_t)(live[c] ? r[c] : 0) * H * K;
-    dr_scales<K>(a, iter, (uint32_t)(a.row0 + r[c]), gain[c]);
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-      gain[c][k] *= dt;
-      p[c][k] = a.x0[k];
-      v[c][k] = a.x0[K + k];
-    }
-  }
-  float ub[S][K];
-#pragma unroll
-  for (int c = 0; c < S; ++c)
-#pragma unroll
-    for (int k = 0; k < K; ++k) ub[c][k] = __ldg(Ub[c] + k);
-  for (int t = 0; t < H; ++t) {
-    const int tn = min(t + 1, H - 1);
-#pragma unroll
-    for (int c = 0; c < S; ++c) {
-      float u[K];
-      float uu = 0.f;
-#pragma unroll
-      for (int k = 0; k < K; ++k) {
-        u[k] = ub[c][k];
-        ub[c][k] = __ldg(Ub[c] + tn * K + k);
-        uu = fmaf(u[k], u[k], uu);
-      }
-      J[c].add(fmaf(pm.w_ctrl, uu, pm_state_cost<K, false>(pm, p[c])), a.kahan);
-#pragma unroll
-      for (int k = 0; k < K; ++k) {
-        v[c][k] = fmaf(gain[c][k], u[k], v[c][k]);
-        p[c][k] = fmaf(dt, v[c][k], p[c][k]);
-      }
-    }
-  }
-#pragma unroll
-  for (int c = 0; c < S; ++c) {
-    J[c].add(pm.w_term * pm_state_cost<K, false>(pm, p[c]), a.kahan);
-    if (live[c]) {
-      float cst = J[c].s;
-      if (!isfinite(cst)) cst = __int_as_float(0x7f800000);
-      a.cost[r[c]] = cst;
-    }
-  }
-}
-
 template <int NL>
 __device__ __forceinline__ void chain_tip(const float (&len)[NL], const float (&c)[NL],
                                           const float (&s)[NL], float& x, float& y) {
@@ -484,86 +318,6 @@ __device__ __forceinline__ bool rollout_chain_body(const RolloutArgs& a, const C
 // Standalone launches: one thread per candidate row.  Direct loads (T = 0)
 // let threads past the last row leave at once; staged loads keep every lane
 // of a warp in the warp's copy protocol.
-template <int K, int T>
-__global__ void __launch_bounds__(kThreads) k_rollout_pm(const RolloutArgs a,
-                                                         const PointMassModel pm) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if constexpr (T == 0) {
-    if (r >= a.rows) return;
-    rollout_pm_body<K, kPrefetchAlone, true, 0>(a, pm, r, true, nullptr);
-  } else {
-    if (__all_sync(0xffffffffu, r >= a.rows)) return;
-    const bool live = r < a.rows;
-    StagedRows<K, T> st;
-    st.init(warp_stage_area(StageShape<K, T>::kWarpBytes), live ? a.U + (size_t)r * a.H * K : nullptr,
-            a.H);
-    rollout_pm_body<K, kPrefetchAlone, true, T>(a, pm, r, live, &st);
-  }
-}
-
-// Rows are padded to whole warps, so a warp belongs to one instance: each
-// warp copies its instance's model (goal, obstacles) to shared memory once.
-// Read from global memory, the obstacle data cost about 6K + 9 loads per
-// step through L1; the standalone kernel reads it as constant operands.
-template <int K, int T>
-__global__ void __launch_bounds__(kThreads) k_rollout_pm_batch(const RolloutArgs* __restrict__ ra,
-                                                               const PointMassModel* __restrict__ pm,
-                                                               const int* __restrict__ row_start,
-                                                               int count) {
-  __shared__ PointMassModel models[kThreads / 32];
-  const int g = blockIdx.x * blockDim.x + threadIdx.x;
-  if (g >= __ldg(row_start + count)) return;  // whole warps: the total is padded to warps
-  const int i = batch_instance(row_start, count, g);
-  PointMassModel& m = models[threadIdx.x >> 5];
-  {
-    const int* src = reinterpret_cast<const int*>(pm + i);
-    int* dst = reinterpret_cast<int*>(&m);
-    for (int w = threadIdx.x & 31; w < (int)(sizeof(PointMassModel) / sizeof(int)); w += 32)
-      dst[w] = __ldg(src + w);
-    __syncwarp();
-  }
-  const RolloutArgs a = ra[i];
-  const int r = g - __ldg(row_start + i);
-  const bool live = r < a.rows;
-  if constexpr (T == 0) {
-    if (!live) return;
-    rollout_pm_body<K, kPrefetchBatch, false, 0>(a, m, r, true, nullptr);
-  } else {
-    StagedRows<K, T> st;
-    st.init(warp_stage_area(StageShape<K, T>::kWarpBytes), live ? a.U + (size_t)r * a.H * K : nullptr,
-            a.H);
-    rollout_pm_body<K, kPrefetchBatch, false, T>(a, m, r, live, &st);
-  }
-}
-
-// Batched point masses, two candidates per thread: instances' rows are
-// padded to 64, and thread g of the launch takes padded rows 64 (g / 32) +
-// (g % 32) and that + 32, which share an instance.
-template <int K>
-__global__ void __launch_bounds__(kThreads) k_rollout_pm_batch2(const RolloutArgs* __restrict__ ra,
-                                                                const PointMassModel* __restrict__ pm,
-                                                                const int* __restrict__ row_start,
-                                                                int count) {
-  __shared__ PointMassModel models[kThreads / 32];
-  const int g = blockIdx.x * blockDim.x + threadIdx.x;
-  const int r0 = (g >> 5) * 64 + (g & 31);
-  if (r0 >= __ldg(row_start + count)) return;  // whole warps: the total is padded to 64
-  const int i = batch_instance(row_start, count, r0);
-  PointMassModel& m = models[threadIdx.x >> 5];
-  {
-    const int* src = reinterpret_cast<const int*>(pm + i);
-    int* dst = reinterpret_cast<int*>(&m);
-    for (int w = threadIdx.x & 31; w < (int)(sizeof(PointMassModel) / sizeof(int)); w += 32)
-      dst[w] = __ldg(src + w);
-    __syncwarp();
-  }
-  const RolloutArgs a = ra[i];
-  const int r[2] = {r0 - __ldg(row_start + i), r0 - __ldg(row_start + i) + 32};
-  const bool live[2] = {r[0] < a.rows, r[1] < a.rows};
-  if (!live[0] && !live[1]) return;
-  rollout_pm_pair<K>(a, m, r, live);
-}
-
 template <int NL, int T>
 __global__ void __launch_bounds__(kThreads) k_rollout_chain(const RolloutArgs a,
                                                             const ChainModel cm) {

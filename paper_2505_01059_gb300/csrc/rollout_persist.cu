@@ -1,6 +1,6 @@
 // rollout_persist.cu -- the rollouts of a whole batch in one persistent
 // launch, or two (Alg. 2 rollout fused with the Eq. 2 cost, the bodies of
-// rollout_kernels.cuh).
+// rollout_kernels.cuh and rollout_pm.cuh).
 //
 // Work items are warp tiles: 32 consecutive candidates of one instance.  The
 // instances are listed group by group, the longest group first and within a
@@ -9,8 +9,8 @@
 // tiles, so item w belongs to the instance whose range holds w.  Each warp of
 // the launch repeatedly takes the next item from a device counter (one
 // atomic add per item), looks its instance up by binary search, and runs
-// that tile's rollout: a point mass of K axes or a planar chain of L links,
-// with direct control loads or staged 4 steps at a time.  A warp therefore
+// that tile's rollout: a point mass of K axes, or a planar chain of L links with
+// direct control loads or staged 4 steps at a time.  A warp therefore
 // moves between instances of different sizes and dynamics, while the warps
 // running at one time mostly run the same body.  The bodies are the
 // per-candidate rollouts of the other kernels (the same templates), so every
@@ -29,8 +29,8 @@
 // CTAs per SM, i.e. at most 170 registers per thread (168 used, no spills).
 //
 // Measured on GB300 on the 256-instance batch (the bench's timed region):
-// 2.68 ms per iteration with two launches, against 2.79-2.91 ms with each
-// group's rollout launched in its own stream's chain.  The order of the
+// 2.43 ms per iteration with two launches (2.68 before the point masses
+// evaluated several steps' costs at once).  The order of the
 // tiles matters: sorted by length alone across all groups, the warps of an
 // SM ran different bodies at once, half of their stall samples were
 // instruction fetches, and the iteration took 3.5 ms; tiles are therefore
@@ -39,34 +39,13 @@
 #include <mutex>
 
 #include "rollout_kernels.cuh"
+#include "rollout_pm.cuh"
 
 namespace mtp {
 namespace {
 
 constexpr int kPersistThreads = 128;
 constexpr int kPersistChunk = 4;  // horizon chunk of a staged tile
-
-// Point masses evaluate every obstacle slot without a branch (ALL): the
-// slots past n_obs add exactly +0, so the bits are those of the guarded loop
-// of the per-group kernel, and mixed with the chains' tiles the branch-free
-// form is faster (256-instance batch 2.73 -> 2.68 ms per iteration).
-template <int K, int T>
-__device__ __forceinline__ bool persist_pm(const RolloutArgs& a, const PointMassModel& m, int r, bool live,
-                                        uint64_t* bars, float* buf, int& seq) {
-  if constexpr (T == 0) {
-    (void)bars;
-    (void)buf;
-    (void)seq;
-    if (!live) return true;
-    return rollout_pm_body<K, kPrefetchBatch, true, 0>(a, m, r, true, nullptr);
-  } else {
-    StagedRows<K, T> st;
-    st.attach(bars, buf, live ? a.U + (size_t)r * a.H * K : nullptr, a.H, seq);
-    const bool ok = rollout_pm_body<K, kPrefetchBatch, true, T>(a, m, r, live, &st);
-    seq = st.seq;
-    return __all_sync(0xffffffffu, ok);
-  }
-}
 
 template <int NL, int T>
 __device__ __forceinline__ bool persist_chain(const RolloutArgs& a, const ChainModel& m, int r, bool live,
@@ -87,15 +66,10 @@ __device__ __forceinline__ bool persist_chain(const RolloutArgs& a, const ChainM
 }
 
 template <int K>
-__device__ __forceinline__ bool pm_tile(int k, bool staged, const RolloutArgs& a, const PointMassModel& m,
-                                        int r, bool live, uint64_t* bars, float* buf, int& seq) {
+__device__ __forceinline__ void pm_item(int k, const RolloutArgs& a, const PointMassModel& m, int r0, float* buf) {
   if constexpr (K <= kPersistMaxAxes) {
-    if (k == K)
-      return staged ? persist_pm<K, kPersistChunk>(a, m, r, live, bars, buf, seq)
-                    : persist_pm<K, 0>(a, m, r, live, bars, buf, seq);
-    return pm_tile<K + 1>(k, staged, a, m, r, live, bars, buf, seq);
-  } else {
-    return false;
+    if (k == K) rollout_pm_lanes<K, PmLane<K>::P, PmLane<K>::T>(a, m, r0, buf);
+    else pm_item<K + 1>(k, a, m, r0, buf);
   }
 }
 
@@ -119,7 +93,7 @@ __global__ void __launch_bounds__(kPersistThreads, 3) k_rollout_persistent(const
   unsigned char* area = persist_smem + (size_t)warp * p.warp_bytes;
   uint64_t* bars = reinterpret_cast<uint64_t*>(area);
   float* buf = reinterpret_cast<float*>(area + 16);
-  if (p.warp_bytes > 0) init_stage_bars(bars);
+  init_stage_bars(bars);
   int seq = 0;
   for (;;) {
     int w = 0;
@@ -137,23 +111,17 @@ __global__ void __launch_bounds__(kPersistThreads, 3) k_rollout_persistent(const
     const int code = __ldg(p.code + lo);
     const int model = __ldg(p.model + lo);
     const RolloutArgs a = p.ra[__ldg(p.order + lo)];
-    const int r = (w - __ldg(p.wstart + lo)) * 32 + lane;
-    const bool live = r < a.rows;
+    const int r0 = (w - __ldg(p.wstart + lo)) * 32;
     const int dim = (code >> 8) & 0xff;
-    // staged only where the instance's rows allow it and this launch has
-    // staging buffers (a direct-load launch has none)
-    const bool staged = p.warp_bytes > 0 && (code >> 16) != 0;
-    bool ok;
+    bool ok = true;
     if ((code & 0xff) == MTP_DYN_POINTMASS) {
-      PointMassModel& m = models[warp];
-      const int* src = reinterpret_cast<const int*>(p.pm + model);
-      int* dst = reinterpret_cast<int*>(&m);
-      for (int q = lane; q < (int)(sizeof(PointMassModel) / sizeof(int)); q += 32) dst[q] = __ldg(src + q);
-      __syncwarp();
-      ok = pm_tile<1>(dim, staged, a, m, r, live, bars, buf, seq);
+      load_pm_model(models[warp], p.pm[model]);
+      pm_item<1>(dim, a, models[warp], r0, buf);
     } else {
+      const int r = r0 + lane;
       const ChainModel cm = p.cm[model];
-      ok = chain_tile<1>(dim, staged, a, cm, r, live, bars, buf, seq);
+      // staged only where the instance's rows allow it and the launch asks for it
+      ok = chain_tile<1>(dim, p.staged && (code >> 16) != 0, a, cm, r, r < a.rows, bars, buf, seq);
     }
     // the model slot and the staging buffers are reused by the next item
     __syncwarp();
@@ -163,16 +131,21 @@ __global__ void __launch_bounds__(kPersistThreads, 3) k_rollout_persistent(const
 
 }  // namespace
 
-size_t persist_warp_bytes(int max_pm_axes_staged, int max_links_staged) {
-  size_t f = 0;
-  auto need = [&](int k) {
-    const int quads = (kPersistChunk * k + 3) / 4;
+template <int K>
+static size_t pm_floats_of(int k) {
+  if constexpr (K <= kPersistMaxAxes) return k == K ? PmLane<K>::floats : pm_floats_of<K + 1>(k);
+  else return 0;
+}
+size_t persist_pm_floats(int axes) { return pm_floats_of<1>(axes); }
+
+size_t persist_warp_bytes(size_t pm_floats, int max_links_staged) {
+  size_t f = pm_floats;
+  if (max_links_staged > 0) {
+    const int quads = (kPersistChunk * max_links_staged + 3) / 4;
     const int stride = 4 * (quads % 2 ? quads : quads + 1);
     f = std::max(f, (size_t)2 * 32 * stride);
-  };
-  if (max_pm_axes_staged > 0) need(max_pm_axes_staged);
-  if (max_links_staged > 0) need(max_links_staged);
-  return f ? 16 + f * sizeof(float) : 0;
+  }
+  return 16 + f * sizeof(float);
 }
 
 int persist_blocks_per_sm(size_t warp_bytes) {
@@ -186,9 +159,9 @@ int persist_blocks_per_sm(size_t warp_bytes) {
   auto it = cache.find({dev, warp_bytes});
   if (it != cache.end()) return it->second;
   // the attribute is the ceiling of every launch's shared memory: the
-  // largest staged tile any batch can have
+  // largest tile any batch can have
   const int warps = kPersistThreads / 32;
-  const size_t ceiling = persist_warp_bytes(kPersistMaxAxes, kPersistMaxLinks) * warps;
+  const size_t ceiling = persist_warp_bytes(kPmLaneFloats, kPersistMaxLinks) * warps;
   if (cudaFuncSetAttribute(k_rollout_persistent, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ceiling) !=
       cudaSuccess)
     return 0;

@@ -146,6 +146,7 @@ struct mtp_batch {
   int device = 0;
   BatchTables t;
   int count = 0;
+  int upd_lanes = 4;                   // lanes per (t, i) element of the updates
   std::vector<BatchGroup> groups;
   // (dyn, n) -> rollout tile chosen by the autotuner: (threads per block, horizon chunk)
   std::map<std::pair<int, int>, std::array<int, 2>> tuned;
@@ -316,6 +317,9 @@ cudaError_t fill_batch(mtp_batch* b, mtp_handle* const* handles, int count, cuda
   // candidate generation, selection and update tables in group order, so
   // that each group's stream launches them over a contiguous range
   hv.d_cand_start[0] = hv.d_z_start[0] = hv.d_local_start[0] = hv.d_warp_start[0] = 0;
+  long long elements = 0;
+  for (int i = 0; i < count; ++i) elements += (long long)handles[i]->dm.H * handles[i]->dm.n;
+  b->upd_lanes = update_lanes(elements);
   std::vector<CandArgs> tc_args(count);
   std::vector<char> is_tc(count, 0);
   for (int pos = 0; pos < count; ++pos) {
@@ -360,7 +364,7 @@ cudaError_t fill_batch(mtp_batch* b, mtp_handle* const* handles, int count, cuda
                                h->elite, h->weight, h->ustar, nullptr, nullptr, h->entropy};
     hv.d_upd[pos] = UpdateArgs{h->U, h->elite, h->weight, dm.E, dm.H, dm.n, h->pr.alpha, h->pr.sigma_min,
                                h->pr.update_rule, h->mu, h->sigma, h->mu_f, h->sigma_f, h->iter_dev};
-    hv.d_warp_start[pos + 1] = hv.d_warp_start[pos] + update_threads(dm.H, dm.n);
+    hv.d_warp_start[pos + 1] = hv.d_warp_start[pos] + update_threads(dm.H, dm.n, b->upd_lanes);
   }
   // tensor-core members, group by group
   {
@@ -630,7 +634,7 @@ cudaError_t enqueue_batch_iteration_persistent(mtp_batch* b, cudaStream_t s, boo
     if (!b->covered[gi]) {
       if ((e = launch_group(b, g, g.block, g.chunk, gs))) return e;
       if ((e = launch_select_batch(t.d_sel + f, g.count, g.sel_smem, gs))) return e;
-      if ((e = launch_update_batch(t.d_upd + f, t.d_warp_start + f, g.count, g.upd_threads, gs))) return e;
+      if ((e = launch_update_batch(t.d_upd + f, t.d_warp_start + f, g.count, g.upd_threads, b->upd_lanes, gs))) return e;
     }
     if ((e = cudaEventRecord(b->group_done[gi], gs))) return e;
   }
@@ -664,7 +668,7 @@ cudaError_t enqueue_batch_iteration_persistent(mtp_batch* b, cudaStream_t s, boo
     const int f = g.first;
     if ((e = cudaStreamWaitEvent(gs, split && !first_part(gi) ? b->persist_ev2 : b->persist_ev, 0))) return e;
     if ((e = launch_select_batch(t.d_sel + f, g.count, g.sel_smem, gs))) return e;
-    if ((e = launch_update_batch(t.d_upd + f, t.d_warp_start + f, g.count, g.upd_threads, gs))) return e;
+    if ((e = launch_update_batch(t.d_upd + f, t.d_warp_start + f, g.count, g.upd_threads, b->upd_lanes, gs))) return e;
     if ((e = cudaEventRecord(b->group_done[gi], gs))) return e;
   }
   for (size_t gi = 0; gi < b->groups.size(); ++gi)
@@ -694,7 +698,7 @@ cudaError_t enqueue_batch_iteration(mtp_batch* b, cudaStream_t s) {
     if ((e = launch_local_batch(t.d_cand + f, t.d_local_start + f, g.count, g.local_blocks, gs))) return e;
     if ((e = launch_group(b, g, g.block, g.chunk, gs))) return e;
     if ((e = launch_select_batch(t.d_sel + f, g.count, g.sel_smem, gs))) return e;
-    if ((e = launch_update_batch(t.d_upd + f, t.d_warp_start + f, g.count, g.upd_threads, gs))) return e;
+    if ((e = launch_update_batch(t.d_upd + f, t.d_warp_start + f, g.count, g.upd_threads, b->upd_lanes, gs))) return e;
     if ((e = cudaEventRecord(b->group_done[gi], gs))) return e;
   }
   for (size_t gi = 0; gi < b->groups.size(); ++gi)

@@ -7,6 +7,8 @@
 // pairs with a bitonic network and computes the softmax weights in FP64.
 // k_update (many CTAs): one warp per (t, i) element reduces the weighted
 // FP64 mean and spread over the elites, applies the floor and the smoothing.
+#include <algorithm>
+
 #include "mtp_device.cuh"
 
 namespace mtp {
@@ -653,7 +655,7 @@ __global__ void __launch_bounds__(kUpdThreads) k_update(const UpdateArgs a) {
 }
 
 // Many planning problems: thread_start (count + 1 entries) holds each
-// instance's first thread.
+// instance's first thread, whole blocks per instance.
 template <int G>
 __global__ void __launch_bounds__(kUpdThreads) k_update_batch(const UpdateArgs* __restrict__ args,
                                                       const int* __restrict__ thread_start,
@@ -748,15 +750,38 @@ cudaError_t launch_select_batch(const SelectArgs* d_args, int count, size_t smem
   return cudaGetLastError();
 }
 
-// Batches have many (t, i) elements: one lane each, no cross-lane sums.
-cudaError_t launch_update_batch(const UpdateArgs* d_args, const int* d_thread_start, int count,
-                                int total_threads, cudaStream_t s) {
-  if (total_threads <= 0) return cudaSuccess;
-  k_update_batch<1><<<(total_threads + kUpdThreads - 1) / kUpdThreads, kUpdThreads, 0, s>>>(d_args, d_thread_start, count);
-  return cudaGetLastError();
+// Lanes per element of a batch's updates, for all its instances' elements: the
+// FP64 pipe, 64 cycles an instruction per SM sub-partition whatever its lanes
+// do, bounds them.  At least 4: with E 64 an element alone takes about 470 FP64
+// instructions, a warp of 32 lane-wide elements therefore 30,000 cycles; 4 lanes
+// per element cut that to a quarter for about 4 % more instructions in all
+// (serving cycle of 48 robots: 48 -> 14 us per group of chains, the cycle 385 ->
+// 345 us).  More lanes while the launch leaves sub-partitions idle.
+int update_lanes(long long elements) {
+  int G = 4;
+  const long long want = (long long)device_sms() * 256;
+  while (G < 32 && elements * G < want) G <<= 1;
+  return G;
 }
 
-int update_threads(int H, int n) { return H * n; }
+// Threads one instance's update gets in a batch: whole blocks.
+int update_threads(int H, int n, int lanes) {
+  const long long threads = std::min<long long>((long long)H * n * lanes, 1 << 18);  // more elements: several sweeps
+  return (int)((threads + kUpdThreads - 1) / kUpdThreads * kUpdThreads);
+}
+
+cudaError_t launch_update_batch(const UpdateArgs* d_args, const int* d_thread_start, int count,
+                                int total_threads, int lanes, cudaStream_t s) {
+  if (total_threads <= 0) return cudaSuccess;
+  const int blocks = total_threads / kUpdThreads;
+  switch (lanes) {
+    case 4: k_update_batch<4><<<blocks, kUpdThreads, 0, s>>>(d_args, d_thread_start, count); break;
+    case 8: k_update_batch<8><<<blocks, kUpdThreads, 0, s>>>(d_args, d_thread_start, count); break;
+    case 16: k_update_batch<16><<<blocks, kUpdThreads, 0, s>>>(d_args, d_thread_start, count); break;
+    default: k_update_batch<32><<<blocks, kUpdThreads, 0, s>>>(d_args, d_thread_start, count); break;
+  }
+  return cudaGetLastError();
+}
 
 // Threads of the single-instance selection block: about kSelKeys keys per
 // thread, at least 128 and at least E (up to 1024), so that with E <= 1024

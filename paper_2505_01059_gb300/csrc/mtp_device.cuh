@@ -335,8 +335,9 @@ cudaError_t launch_rollout_chain_batch(const RolloutArgs* d_ra, const ChainModel
                                        int links, int block, int chunk, cudaStream_t s);
 cudaError_t launch_select_batch(const SelectArgs* d_args, int count, size_t smem, cudaStream_t s);
 cudaError_t launch_update_batch(const UpdateArgs* d_args, const int* d_thread_start, int count,
-                                int total_threads, cudaStream_t s);
-int update_threads(int H, int n);  // threads one instance's update gets in a batch
+                                int total_threads, int lanes, cudaStream_t s);
+int update_lanes(long long elements);         // lanes per (t, i) element of a batch's updates
+int update_threads(int H, int n, int lanes);  // threads one instance's update gets in a batch
 cudaError_t launch_scatter(const float* packed, float* const* d_dst, const int* d_off, int count,
                            cudaStream_t s);
 cudaError_t launch_gather(const float* const* d_src, const int* d_off, float* packed, int count,

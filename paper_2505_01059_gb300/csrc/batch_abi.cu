@@ -35,7 +35,7 @@ struct BatchGroup {
   // entries [tc_first, tc_first + tc_count) of the tensor-core argument list,
   // their tile numbering at tc_start_first of d_tc_start
   int tc_first = 0, tc_count = 0, tc_start_first = 0, tc_tiles = 0;
-  size_t cand_smem = 0, sel_smem = 0;
+  size_t cand_smem = 0, sel_smem = 0, tc_smem = 0;
   double est = 0.0;  // expected rollout time (ms): sets the groups' launch order
 };
 
@@ -373,11 +373,13 @@ cudaError_t fill_batch(mtp_batch* b, mtp_handle* const* handles, int count, cuda
       g.tc_first = tc_pos;
       g.tc_start_first = seg;
       int tiles = 0;
+      g.tc_smem = 0;
       hv.d_tc_start[seg] = 0;
       for (int pos = g.first; pos < g.first + g.count; ++pos) {
         if (!is_tc[pos]) continue;
         hv.d_tc[tc_pos++] = tc_args[pos];
         tiles += bspline_tc_tiles(tc_args[pos]);
+        g.tc_smem = std::max(g.tc_smem, bspline_tc_smem(tc_args[pos]));
         hv.d_tc_start[seg + (tc_pos - g.tc_first)] = tiles;
       }
       g.tc_count = tc_pos - g.tc_first;
@@ -628,7 +630,7 @@ cudaError_t enqueue_batch_iteration_persistent(mtp_batch* b, cudaStream_t s, boo
       return e;
     if (g.tc_count > 0 &&
         (e = launch_bspline_tc_batch(t.d_tc + g.tc_first, t.d_tc_start + g.tc_start_first, g.tc_count,
-                                     g.tc_tiles, gs)))
+                                     g.tc_tiles, g.tc_smem, gs)))
       return e;
     if ((e = launch_local_batch(t.d_cand + f, t.d_local_start + f, g.count, g.local_blocks, gs))) return e;
     if (!b->covered[gi]) {
@@ -693,7 +695,7 @@ cudaError_t enqueue_batch_iteration(mtp_batch* b, cudaStream_t s) {
       return e;
     if (g.tc_count > 0 &&
         (e = launch_bspline_tc_batch(t.d_tc + g.tc_first, t.d_tc_start + g.tc_start_first, g.tc_count,
-                                     g.tc_tiles, gs)))
+                                     g.tc_tiles, g.tc_smem, gs)))
       return e;
     if ((e = launch_local_batch(t.d_cand + f, t.d_local_start + f, g.count, g.local_blocks, gs))) return e;
     if ((e = launch_group(b, g, g.block, g.chunk, gs))) return e;

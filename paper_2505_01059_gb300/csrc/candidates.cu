@@ -402,8 +402,9 @@ __global__ void __launch_bounds__(kThreads) k_local_batch(const CandArgs* __rest
   local_rows_body<kLocalFull>(args[lo], blk - local_start[lo], local_start[lo + 1] - local_start[lo]);
 }
 
-// Def. 1: the graph Z of the current iteration written to global memory,
-// block `blk` of `nblk` given to it, four dimensions per generator call.
+// Def. 1: the graph Z of the current iteration written to global memory (in
+// bfloat16 for the tensor cores), block `blk` of `nblk` given to it, four
+// dimensions per generator call.
 __device__ __forceinline__ void graph_Z_body(const CandArgs& a, float* Z, int blk, int nblk) {
   __shared__ float box_lo[MTP_MAX_CTRL], box_hi[MTP_MAX_CTRL];
   stage_box(a, box_lo, box_hi);
@@ -416,7 +417,10 @@ __device__ __forceinline__ void graph_Z_body(const CandArgs& a, float* Z, int bl
 #pragma unroll
     for (int w = 0; w < 4; ++w) {
       const int i = 4 * g + w;
-      if (i < n) Z[node * n + i] = fmaf(box_hi[i] - box_lo[i], unit24(pick(r, w)), box_lo[i]);
+      if (i >= n) continue;
+      const float z = fmaf(box_hi[i] - box_lo[i], unit24(pick(r, w)), box_lo[i]);
+      if (a.basis_tc) reinterpret_cast<__nv_bfloat16*>(Z)[node * n + i] = __float2bfloat16_rn(z);
+      else Z[node * n + i] = z;
     }
   }
 }

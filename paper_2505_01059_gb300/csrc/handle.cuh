@@ -16,6 +16,7 @@ struct mtp_handle {
   mtp::Key key{};
   // interpolation tables
   float* basis = nullptr;
+  uint16_t* basis_tc = nullptr;  // the basis as tensor-core operands (tc_graph)
   int32_t* bfirst = nullptr;
   int32_t* seg = nullptr;
   float* delta = nullptr;
@@ -55,7 +56,7 @@ struct mtp_handle {
   double* weight = nullptr;
   float* ustar = nullptr;
   float* x0 = nullptr;
-  float* Z = nullptr;  // (M, N, n) graph of the current iteration (batched planning)
+  float* Z = nullptr;  // (M, N, n) graph of the current iteration (bfloat16 when tc_graph)
   uint32_t* status = nullptr;  // device status word: bits a rollout sets when a bounded wait gave up
   int rollout_chunk = 0;       // horizon chunk of the staged control loads of a lone rollout (0: direct)
   bool tc_graph = false;       // graph rows contracted on the tensor cores (BF16 B-spline)

@@ -212,6 +212,11 @@ mtp_status build_tables(mtp_handle* h) {
     }
   }
   MTP_CUDA(h, dalloc(&h->basis, basis.size()));
+  if (h->tc_graph) {
+    const std::vector<uint16_t> tc = bspline_tc_basis(basis.data(), H, M);
+    MTP_CUDA(h, dalloc(&h->basis_tc, tc.size()));
+    MTP_CUDA(h, cudaMemcpy(h->basis_tc, tc.data(), tc.size() * 2, cudaMemcpyHostToDevice));
+  }
   MTP_CUDA(h, dalloc(&h->bfirst, H));
   MTP_CUDA(h, dalloc(&h->seg, H));
   MTP_CUDA(h, dalloc(&h->delta, H));
@@ -252,6 +257,7 @@ CandArgs cand_args(const mtp_handle* h, uint32_t iter, const uint32_t* d_iter) {
   a.bf16 = (h->pr.flags & MTP_FLAG_BF16_BASIS) ? 1 : 0;
   a.inv_h = h->inv_h;
   a.basis = h->basis;
+  a.basis_tc = h->basis_tc;
   a.bfirst = h->bfirst;
   a.seg = h->seg;
   a.delta = h->delta;
@@ -652,7 +658,7 @@ void free_handle(mtp_handle* h) {
   if (h->side) cudaStreamDestroy(h->side);
   if (h->ev_fork) cudaEventDestroy(h->ev_fork);
   if (h->ev_join) cudaEventDestroy(h->ev_join);
-  void* ptrs[] = {h->basis, h->bfirst, h->seg, h->delta, h->mu, h->sigma, h->mu_f, h->sigma_f,
+  void* ptrs[] = {h->basis, h->basis_tc, h->bfirst, h->seg, h->delta, h->mu, h->sigma, h->mu_f, h->sigma_f,
                   h->iter_dev,
                   h->Ubuf[0], h->Ubuf[1], h->cost, h->elite, h->weight, h->ustar, h->x0, h->Z,
                   h->status, h->entropy, h->sel_pairs};
@@ -706,7 +712,8 @@ mtp_status mtp_create(const mtp_problem* problem, mtp_handle** out) {
       (e = dalloc(&h->iter_dev, 1)) || (e = dalloc(&h->Ubuf[0], rowsz * dm.B)) ||
       (e = dalloc(&h->cost, dm.B)) || (e = dalloc(&h->elite, dm.E)) ||
       (e = dalloc(&h->weight, dm.E)) || (e = dalloc(&h->ustar, dm.n)) ||
-      (e = dalloc(&h->x0, dm.d)) || (e = dalloc(&h->Z, (size_t)dm.M * dm.N * dm.n)) ||
+      (e = dalloc(&h->x0, dm.d)) ||
+      (e = dalloc(&h->Z, ((size_t)dm.M * dm.N * dm.n + 7) / 8 * 8)) ||  // whole 16-byte pieces as bfloat16 too
       (e = dalloc(&h->status, 1)) ||
       ((p.flags & MTP_FLAG_COST_ENTROPY) && (e = dalloc(&h->entropy, 1))) ||
       (h->sel_chunks > 0 && (e = dalloc(&h->sel_pairs, (size_t)h->sel_chunks * dm.E))))
@@ -749,6 +756,8 @@ mtp_status mtp_problem_device_bytes(const mtp_problem* problem, uint64_t* bytes)
     if (chunks > 0) *bytes += r((uint64_t)chunks * p.E * 8);          // selection pairs
   }
   const Dims dm = dims_of(p);
+  if (tc_graph_rule(p, dm))
+    *bytes += r((uint64_t)((p.horizon + 127) / 128) * 128 * ((p.M + 15) / 16 * 16) * 2);  // tensor-core basis
   bool on = false, local = false;
   int grid = 0;
   size_t smem = 0;

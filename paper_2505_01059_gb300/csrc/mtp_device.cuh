@@ -4,6 +4,7 @@
 
 #include <cstdint>
 #include <string>
+#include <vector>
 
 #include <cuda_runtime.h>
 
@@ -64,8 +65,11 @@ __device__ __forceinline__ int32_t index_of(uint32_t r, uint32_t N) {
   return (int32_t)__umulhi(r, N);
 }
 
+// v inside the box; NaN stays NaN.
 __device__ __forceinline__ float clamp_box(float v, float lo, float hi) {
-  return v < lo ? lo : (v > hi ? hi : v);
+  float r;
+  asm("{\n .reg .f32 t;\n max.NaN.f32 t, %1, %2;\n min.NaN.f32 %0, t, %3;\n}" : "=f"(r) : "f"(v), "f"(lo), "f"(hi));
+  return r;
 }
 
 // Compensated (Kahan) accumulation in FP32.
@@ -119,6 +123,8 @@ struct CandArgs {
                            // rounded on the host, the knots as they are gathered)
   float inv_h;             // reciprocal knot spacing of the Akima / linear knots
   const float* basis;      // (H, M) B-spline basis, row t
+  const uint16_t* basis_tc; // the same as the tensor cores' B operands (bspline_tc_basis), when
+                           // the graph rows go there; Z_global then holds bfloat16 values
   const int32_t* bfirst;   // (H) first non-zero basis column of row t
   const int32_t* seg;      // (H) Akima / linear piece of step t
   const float* delta;      // (H) offset of step t from the piece's left knot
@@ -299,8 +305,10 @@ bool bspline_tc_eligible(const CandArgs& a);
 int bspline_tc_tiles(const CandArgs& a);
 cudaError_t init_bspline_tc_attributes();
 cudaError_t launch_bspline_tc(const CandArgs& a, cudaStream_t s);
+std::vector<uint16_t> bspline_tc_basis(const float* basis, int H, int M);
+size_t bspline_tc_smem(const CandArgs& a);  // shared memory of a CTA on that instance
 cudaError_t launch_bspline_tc_batch(const CandArgs* d_args, const int* d_tile_start, int count,
-                                    int total_tiles, cudaStream_t s);
+                                    int total_tiles, size_t smem, cudaStream_t s);
 cudaError_t launch_select(const SelectArgs& a, cudaStream_t s);
 // Two-stage selection for B beyond one block: chunks > 0 stages of `chunk`
 // costs each (select_plan; chunks = 0: one block suffices, -1: too large).

@@ -39,12 +39,12 @@ __device__ __forceinline__ float akima_knot_slope(int a, int M, SlopeFn slope) {
 // 2 pi u2 is evaluated as pi + x with x = 2 pi (u2 - 1/2) in [-pi, pi), where
 // the SFU sine / cosine have absolute error about 4e-7; the radius keeps the
 // accurate logarithm because it is ill-conditioned for u1 near 1.  Its
-// square root is r2 * rsqrt(r2) (a few ulp; r2 = 0 when u1 = 1).
+// square root is r2 * rsqrt(r2) (a few ulp), the argument kept normal: 0 when u1 = 1.
 __device__ __forceinline__ void box_muller(uint32_t w0, uint32_t w1, float& e0, float& e1) {
   const float u1 = (float)((w0 >> 8) + 1u) * 5.9604644775390625e-8f;  // (0, 1]
   const float u2 = (float)(w1 >> 8) * 5.9604644775390625e-8f;         // [0, 1)
-  const float r2 = -2.f * logf(u1);
-  const float radius = r2 > 0.f ? r2 * rsqrtf(r2) : 0.f;
+  const float r2 = -2.f * logf(u1);  // 0, or at least 2^-24
+  const float radius = r2 * rsqrt_normal(fmaxf(r2, kMinNormal));
   float sn, cs;
   __sincosf(6.28318530717958648f * (u2 - 0.5f), &sn, &cs);
   e0 = -radius * cs;
@@ -85,7 +85,7 @@ __device__ __forceinline__ void local_rows_body(const CandArgs& a, int lb, int n
   float* __restrict__ const U_mean = a.U_mean;
   const float* __restrict__ const mu = a.mu;
   const float* __restrict__ const sigma = a.sigma;
-  const Key key = a.key;
+  const RoundKeys keys = a.round_keys;
   const int rows = local_rows + ((MODE != kLocalNoise && U_mean) ? 1 : 0);  // + the mean row
   // whole 16-byte groups: one vector load of mu and sigma and one vector
   // store per generator call (rows of a 16-byte aligned tensor stay aligned)
@@ -127,7 +127,7 @@ __device__ __forceinline__ void local_rows_body(const CandArgs& a, int lb, int n
             for (int w = 0; w < 4; ++w) eps[w] = (4 * q + w < Hn) ? dst[4 * q + w] : 0.f;
           }
         } else {
-          const uint4 r = philox(make_uint4((uint32_t)row, (uint32_t)q, iter, kTagLocal), key);
+          const uint4 r = philox(make_uint4((uint32_t)row, (uint32_t)q, iter, kTagLocal), keys);
           box_muller(r.x, r.y, eps[0], eps[1]);
           box_muller(r.z, r.w, eps[2], eps[3]);
         }
@@ -337,36 +337,31 @@ __device__ __forceinline__ void graph_paths_body(const CandArgs& a, const float*
   }
 }
 
-// One block of candidate generation for one planning problem: block `bid`
-// of `nblocks` blocks that instance is given (graph blocks first).
-__device__ __forceinline__ void candidates_body(const CandArgs& a, float* smem, int bid,
-                                                int nblocks) {
-  if (bid < a.graph_blocks) {
-    __shared__ float box_lo[MTP_MAX_CTRL], box_hi[MTP_MAX_CTRL];
-    stage_box(a, box_lo, box_hi);
-    const uint32_t iter = (a.d_iter ? *a.d_iter : a.iter) + a.iter_offset;
-    float* Z = smem;
-    float* C = Z + ((a.C_in || a.Z_global) ? 0 : a.dm.M * a.dm.N * a.dm.n);
-    const float* Zs = a.Z_global;
-    if (a.C_in == nullptr && Zs == nullptr) {
-      regenerate_Z(a, Z, iter, box_lo, box_hi);
-      __syncthreads();
-      Zs = Z;
-    }
-    graph_paths_body(a, Zs, C, bid, iter, box_lo, box_hi);
-    return;
+// Graph block `bid` of one planning problem.
+__device__ __forceinline__ void graph_block_body(const CandArgs& a, float* smem, int bid) {
+  __shared__ float box_lo[MTP_MAX_CTRL], box_hi[MTP_MAX_CTRL];
+  stage_box(a, box_lo, box_hi);
+  const uint32_t iter = (a.d_iter ? *a.d_iter : a.iter) + a.iter_offset;
+  float* Z = smem;
+  float* C = Z + ((a.C_in || a.Z_global) ? 0 : a.dm.M * a.dm.N * a.dm.n);
+  const float* Zs = a.Z_global;
+  if (a.C_in == nullptr && Zs == nullptr) {
+    regenerate_Z(a, Z, iter, box_lo, box_hi);
+    __syncthreads();
+    Zs = Z;
   }
-  local_rows_body<kLocalFull>(a, bid - a.graph_blocks, nblocks - a.graph_blocks);
+  graph_paths_body(a, Zs, C, bid, iter, box_lo, box_hi);
 }
 
 __global__ void __launch_bounds__(kThreads, 5) k_candidates(const CandArgs a) {
   extern __shared__ float smem[];
-  candidates_body(a, smem, blockIdx.x, gridDim.x);
+  if ((int)blockIdx.x < a.graph_blocks) graph_block_body(a, smem, blockIdx.x);
+  else local_rows_body<kLocalFull>(a, (int)blockIdx.x - a.graph_blocks, (int)gridDim.x - a.graph_blocks);
 }
 
-// Many planning problems in one launch: block_start (count + 1 entries)
-// gives each instance's first block; each block copies its instance's
-// arguments into shared memory and runs the same body.
+// The graph blocks of many planning problems in one launch: block_start (count
+// + 1 entries) gives each instance's first block; each block copies its
+// instance's arguments into shared memory and runs the same body.
 __global__ void __launch_bounds__(kThreads) k_candidates_batch(const CandArgs* __restrict__ args,
                                                                const int* __restrict__ block_start,
                                                                int count) {
@@ -383,7 +378,7 @@ __global__ void __launch_bounds__(kThreads) k_candidates_batch(const CandArgs* _
   int* dst = reinterpret_cast<int*>(&sa);
   for (int w = threadIdx.x; w < (int)(sizeof(CandArgs) / sizeof(int)); w += blockDim.x) dst[w] = src[w];
   __syncthreads();
-  candidates_body(sa, smem, blk - block_start[lo], block_start[lo + 1] - block_start[lo]);
+  graph_block_body(sa, smem, blk - block_start[lo]);
 }
 
 // Local rows of many planning problems (no shared memory, so the blocks

@@ -250,6 +250,7 @@ CandArgs cand_args(const mtp_handle* h, uint32_t iter, const uint32_t* d_iter) {
   CandArgs a{};
   a.dm = h->dm;
   a.key = h->key;
+  a.round_keys = round_keys(h->key);
   a.iter = iter;
   a.d_iter = d_iter;
   a.interp = h->pr.interp;

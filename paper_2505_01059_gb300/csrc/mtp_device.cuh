@@ -45,6 +45,29 @@ __device__ __forceinline__ uint4 philox(uint4 c, Key key) {
   return c;
 }
 
+// The generator's ten round keys: the key, bumped by the Weyl constants.
+struct RoundKeys {
+  Key k[10];
+};
+inline RoundKeys round_keys(Key key) {
+  RoundKeys r;
+  for (uint32_t i = 0; i < 10; ++i) r.k[i] = Key{key.k0 + i * 0x9E3779B9u, key.k1 + i * 0xBB67AE85u};
+  return r;
+}
+
+// The same with the round keys made ahead: read from a kernel's parameters they
+// are operands of the rounds' exclusive-ors, and each round is four instructions.
+__device__ __forceinline__ uint4 philox(uint4 c, const RoundKeys& rk) {
+#pragma unroll
+  for (int r = 0; r < 10; ++r) {
+    const unsigned long long p0 = 0xD2511F53ull * c.x, p1 = 0xCD9E8D57ull * c.z;
+    const uint32_t lo0 = (uint32_t)p0, hi0 = (uint32_t)(p0 >> 32);
+    const uint32_t lo1 = (uint32_t)p1, hi1 = (uint32_t)(p1 >> 32);
+    c = make_uint4(hi1 ^ c.y ^ rk.k[r].k0, lo1, hi0 ^ c.w ^ rk.k[r].k1, lo0);
+  }
+  return c;
+}
+
 __device__ __forceinline__ uint32_t pick(uint4 v, uint32_t w) {
   return w == 0 ? v.x : (w == 1 ? v.y : (w == 2 ? v.z : v.w));
 }
@@ -71,6 +94,16 @@ __device__ __forceinline__ float clamp_box(float v, float lo, float hi) {
   asm("{\n .reg .f32 t;\n max.NaN.f32 t, %1, %2;\n min.NaN.f32 %0, t, %3;\n}" : "=f"(r) : "f"(v), "f"(lo), "f"(hi));
   return r;
 }
+
+// 1 / sqrt(x) of a normal x (the SFU's value, as rsqrtf gives it there, without
+// the rescaling that covers subnormal arguments: a latency of 18 cycles instead
+// of 41, one instruction instead of four).
+__device__ __forceinline__ float rsqrt_normal(float x) {
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+constexpr float kMinNormal = 1.17549435e-38f;
 
 // Compensated (Kahan) accumulation in FP32.
 struct KahanSum {
@@ -113,6 +146,7 @@ enum LocalMode : int32_t { kLocalFull = 0, kLocalNoise = 1, kLocalFinish = 2 };
 struct CandArgs {
   Dims dm;
   Key key;
+  RoundKeys round_keys;    // the key's, for the local rows
   uint32_t iter;
   const uint32_t* d_iter;  // when set, the iteration is read from here
   uint32_t iter_offset;    // added to that iteration (1: the next iteration's draws)

@@ -37,14 +37,6 @@ constexpr int kPmThreads = 128;  // at most four warps per block
 constexpr int kMaxPmAxes = 16;
 constexpr int kPmSmemMax = 68 * 1024;  // dynamic shared memory of a block, at most
 
-// 1 / sqrt(x) of a normal x (the SFU's value, as rsqrtf gives it there, without
-// the rescaling that covers subnormal arguments: 18 cycles instead of 41).
-__device__ __forceinline__ float rsqrt_normal(float x) {
-  float r;
-  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
-}
-
 __device__ __forceinline__ void copy_async_16(float* smem_dst, const float* gmem_src) {
   const unsigned dst = (unsigned)__cvta_generic_to_shared(smem_dst);
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(gmem_src) : "memory");
@@ -113,7 +105,7 @@ __device__ __forceinline__ void pm_state_costs(const PointMassModel& pm, const f
       const float r = pm.obs_r[o + z];
 #pragma unroll
       for (int j = 0; j < P; ++j) {
-        const float dist = __fmul_rn(d2[z][j], rsqrt_normal(fmaxf(d2[z][j], 1.17549435e-38f)));
+        const float dist = __fmul_rn(d2[z][j], rsqrt_normal(fmaxf(d2[z][j], kMinNormal)));
         pen[j] += fmaxf(r - dist, 0.f);
       }
     }

@@ -58,7 +58,11 @@ constexpr int kPersistFirstFewer = MTP_PERSIST_FIRST_FEWER;
 // Horizon chunk of staged control loads before the autotuner has run.
 constexpr int kDefaultChunk = 4;
 constexpr size_t kBatchGraphSmem = 40 * 1024;  // four graph blocks per SM
-constexpr int kLocalRowsPerThreadBatch = 16;
+// Groups of four elements per thread of the local rows, each thread on one q
+// group of several rows, so that its set-up (instance search, box, the group's
+// mean and spread) is paid once for them: up to 32 (the batch of 256: 4 / 8 / 16 /
+// 32: 2.42 / 2.30 / 2.25 / 2.22 ms), fewer where the launch would leave SMs idle.
+constexpr int kLocalRowsPerThreadBatch = 32;
 
 // Device tables of a batch, packed into one device block that is refilled in
 // place from a pinned host mirror with one copy.  The layout depends on the
@@ -320,6 +324,12 @@ cudaError_t fill_batch(mtp_batch* b, mtp_handle* const* handles, int count, cuda
   long long elements = 0;
   for (int i = 0; i < count; ++i) elements += (long long)handles[i]->dm.H * handles[i]->dm.n;
   b->upd_lanes = update_lanes(elements);
+  long long local_items = 0;
+  for (int i = 0; i < count; ++i)
+    local_items += ((long long)handles[i]->dm.L + 1) * (((long long)handles[i]->dm.H * handles[i]->dm.n + 3) / 4);
+  int local_rows_per_thread = kLocalRowsPerThreadBatch;
+  while (local_rows_per_thread > 4 && local_items < 256LL * local_rows_per_thread * 8 * device_sms())
+    local_rows_per_thread /= 2;
   std::vector<CandArgs> tc_args(count);
   std::vector<char> is_tc(count, 0);
   for (int pos = 0; pos < count; ++pos) {
@@ -355,11 +365,11 @@ cudaError_t fill_batch(mtp_batch* b, mtp_handle* const* handles, int count, cuda
     const long long items = ((long long)dm.L + 1) * (((long long)Hn + 3) / 4);
     hv.d_cand[pos] = c;
     hv.d_cand_start[pos + 1] = hv.d_cand_start[pos] + c.graph_blocks;  // local rows run apart
-    // 16 groups of four elements per thread: each thread's set-up (instance
-    // search, box, its group's mean and spread) is paid once for 16 rows
+    // 32 groups of four elements per thread: each thread's set-up (instance
+    // search, box, its group's mean and spread) is paid once for 32 rows (4 / 8 / 16 / 32: 2.42 / 2.30 / 2.25 / 2.22 ms)
     hv.d_local_start[pos + 1] =
-        hv.d_local_start[pos] + (int)std::max<long long>(1, (items + 256 * kLocalRowsPerThreadBatch - 1) /
-                                                                (256 * kLocalRowsPerThreadBatch));
+        hv.d_local_start[pos] + (int)std::max<long long>(1, (items + 256 * local_rows_per_thread - 1) /
+                                                                (256 * local_rows_per_thread));
     hv.d_sel[pos] = SelectArgs{h->cost, h->U, dm.B, dm.E, dm.H, dm.n, 1.0 / h->pr.lambda, h->pr.update_rule,
                                h->elite, h->weight, h->ustar, nullptr, nullptr, h->entropy};
     hv.d_upd[pos] = UpdateArgs{h->U, h->elite, h->weight, dm.E, dm.H, dm.n, h->pr.alpha, h->pr.sigma_min,

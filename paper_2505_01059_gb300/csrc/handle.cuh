@@ -18,8 +18,7 @@ struct mtp_handle {
   float* basis = nullptr;
   uint16_t* basis_tc = nullptr;  // the basis as tensor-core operands (tc_graph)
   int32_t* bfirst = nullptr;
-  int32_t* seg = nullptr;
-  float* delta = nullptr;
+  float2* piece = nullptr;
   float inv_h = 1.f;
   int paths_per_block = 1;
   bool global_Z = false;  // Z written once per iteration instead of per graph block

@@ -174,8 +174,8 @@ mtp_status build_tables(mtp_handle* h) {
   const bool bf16 = (p.flags & MTP_FLAG_BF16_BASIS) != 0;
   const int H = p.horizon, M = p.M;
   std::vector<float> basis((size_t)H * M, 0.f);
-  std::vector<int32_t> bfirst(H, 0), seg(H, 0);
-  std::vector<float> delta(H, 0.f);
+  std::vector<int32_t> bfirst(H, 0);
+  std::vector<float2> piece(H, make_float2(0.f, 0.f));
   if (p.interp == MTP_INTERP_BSPLINE) {
     const int deg = p.bspline_degree;
     for (int j = 0; j < H; ++j) {
@@ -207,8 +207,9 @@ mtp_status build_tables(mtp_handle* h) {
       if (k > M - 2) k = M - 2;
       const double t = lit ? (double)j / (double)H : (H > 1 ? (double)j / (double)(H - 1) : 0.0);
       const double tk = lit ? (double)k / (double)M : (double)k / (double)(M - 1);
-      seg[j] = (int32_t)k;
-      delta[j] = (float)(t - tk);
+      const int32_t k32 = (int32_t)k;
+      std::memcpy(&piece[j].x, &k32, 4);
+      piece[j].y = (float)(t - tk);
     }
   }
   MTP_CUDA(h, dalloc(&h->basis, basis.size()));
@@ -218,12 +219,10 @@ mtp_status build_tables(mtp_handle* h) {
     MTP_CUDA(h, cudaMemcpy(h->basis_tc, tc.data(), tc.size() * 2, cudaMemcpyHostToDevice));
   }
   MTP_CUDA(h, dalloc(&h->bfirst, H));
-  MTP_CUDA(h, dalloc(&h->seg, H));
-  MTP_CUDA(h, dalloc(&h->delta, H));
+  MTP_CUDA(h, dalloc(&h->piece, H));
   MTP_CUDA(h, cudaMemcpy(h->basis, basis.data(), basis.size() * 4, cudaMemcpyHostToDevice));
   MTP_CUDA(h, cudaMemcpy(h->bfirst, bfirst.data(), H * 4, cudaMemcpyHostToDevice));
-  MTP_CUDA(h, cudaMemcpy(h->seg, seg.data(), H * 4, cudaMemcpyHostToDevice));
-  MTP_CUDA(h, cudaMemcpy(h->delta, delta.data(), H * 4, cudaMemcpyHostToDevice));
+  MTP_CUDA(h, cudaMemcpy(h->piece, piece.data(), H * sizeof(float2), cudaMemcpyHostToDevice));
   return MTP_OK;
 }
 
@@ -260,8 +259,7 @@ CandArgs cand_args(const mtp_handle* h, uint32_t iter, const uint32_t* d_iter) {
   a.basis = h->basis;
   a.basis_tc = h->basis_tc;
   a.bfirst = h->bfirst;
-  a.seg = h->seg;
-  a.delta = h->delta;
+  a.piece = h->piece;
   a.paths_per_block = h->paths_per_block;
   a.mu = h->mu_f;
   a.sigma = h->sigma_f;
@@ -659,7 +657,7 @@ void free_handle(mtp_handle* h) {
   if (h->side) cudaStreamDestroy(h->side);
   if (h->ev_fork) cudaEventDestroy(h->ev_fork);
   if (h->ev_join) cudaEventDestroy(h->ev_join);
-  void* ptrs[] = {h->basis, h->basis_tc, h->bfirst, h->seg, h->delta, h->mu, h->sigma, h->mu_f, h->sigma_f,
+  void* ptrs[] = {h->basis, h->basis_tc, h->bfirst, h->piece, h->mu, h->sigma, h->mu_f, h->sigma_f,
                   h->iter_dev,
                   h->Ubuf[0], h->Ubuf[1], h->cost, h->elite, h->weight, h->ustar, h->x0, h->Z,
                   h->status, h->entropy, h->sel_pairs};
@@ -743,7 +741,7 @@ mtp_status mtp_problem_device_bytes(const mtp_problem* problem, uint64_t* bytes)
   const mtp_problem p = normalized(*problem);
   const uint64_t rowsz = (uint64_t)p.horizon * p.ctrl_dim;
   auto r = [](uint64_t b) { return (b + 511) & ~uint64_t(511); };  // allocation granularity
-  *bytes = r((uint64_t)p.horizon * p.M * 4) + 3 * r((uint64_t)p.horizon * 4)  // tables
+  *bytes = r((uint64_t)p.horizon * p.M * 4) + r((uint64_t)p.horizon * 4) + r((uint64_t)p.horizon * 8)  // tables
            + 2 * r(rowsz * 8) + 2 * r(rowsz * 4) + r(4)                       // mean, spread
            + r(rowsz * p.B * 4) + r((uint64_t)p.B * 4)                        // U, cost
            + r((uint64_t)p.E * 4) + r((uint64_t)p.E * 8)                      // elites, weights

@@ -160,8 +160,8 @@ struct CandArgs {
   const uint16_t* basis_tc; // the same as the tensor cores' B operands (bspline_tc_basis), when
                            // the graph rows go there; Z_global then holds bfloat16 values
   const int32_t* bfirst;   // (H) first non-zero basis column of row t
-  const int32_t* seg;      // (H) Akima / linear piece of step t
-  const float* delta;      // (H) offset of step t from the piece's left knot
+  const float2* piece;     // (H) Akima / linear piece of step t (the bits of a whole number) and
+                           // the step's offset from the piece's left knot
   // graph rows
   const float* C_in;       // (P, M, n) given waypoints, or null to sample them
   const float* Z_global;   // (M, N, n) graph already in global memory, or null to

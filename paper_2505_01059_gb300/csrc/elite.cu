@@ -1,10 +1,11 @@
 // elite.cu -- Alg. 2 elite selection and the modified CEM update.
 //
 // k_select (one CTA): turns the B costs into order-preserving 32-bit keys
-// (NaN -> +inf, -0 -> +0), finds the E-th smallest key by a 4-pass 8-bit
-// radix select over shared memory, collects the keys below it plus the
-// lowest-index ties (a block scan in index order), sorts those E (key, index)
-// pairs with a bitonic network and computes the softmax weights in FP64.
+// (NaN -> +inf, -0 -> +0), narrows the bin of the E-th smallest key by 8-bit
+// radix passes over shared memory, collects the keys below it and the bin's (or
+// its lowest-index ties, a block scan in index order), orders those (key, index)
+// pairs (each counts the smaller ones, or a bitonic network for many elites) and
+// computes the softmax weights in FP64.
 // k_update (many CTAs): one warp per (t, i) element reduces the weighted
 // FP64 mean and spread over the elites, applies the floor and the smoothing.
 #include <algorithm>
@@ -17,7 +18,8 @@ namespace {
 constexpr int kSelThreads = 1024;
 constexpr size_t kSelSmemMax = 200 * 1024;  // dynamic shared memory of one selection block
 constexpr int kOneBlockMax = 32768;         // above this, two stages (measured below)
-constexpr int kChunkKeys = 16384;           // first-stage chunk length
+constexpr int kChunkKeys = 16384;           // first-stage chunk length, at most
+constexpr int kChunkLeast = 4096;           // and at least
 
 __device__ __forceinline__ uint32_t order_key(float f) {
   if (isnan(f)) f = __int_as_float(0x7f800000);
@@ -32,11 +34,14 @@ __device__ __forceinline__ float key_cost(uint32_t k) {
   return __uint_as_float((k & 0x80000000u) ? (k & 0x7fffffffu) : ~k);
 }
 
-__device__ __forceinline__ int next_pow2(int v) {
+__host__ __device__ __forceinline__ int next_pow2(int v) {
   int p = 1;
   while (p < v) p <<= 1;
   return p;
 }
+
+// At most this many elites are ordered by counting, with a softmax of a warp or two.
+constexpr int kFewElites = 64;
 
 // Bins with at most this many keys end the radix passes early.
 constexpr int kBoundaryMax = 64;
@@ -46,25 +51,42 @@ constexpr int kBoundaryMax = 64;
 // plain loop: batched, the 7-link arm's two passes took 3.0 us instead of 2.3).
 constexpr int kSelBatch = 8;
 
-// Ascending bitonic sort of 64 values held two per lane (v0 = element lane,
-// v1 = element lane + 32) in one warp.
-__device__ __forceinline__ void warp_sort64(unsigned long long& v0, unsigned long long& v1, int lane) {
-  for (int k = 2; k <= 64; k <<= 1) {
-    for (int j = k >> 1; j > 0; j >>= 1) {
-      if (j == 32) {  // partner is the lane's other element (k == 64, ascending)
-        const unsigned long long lo = v0 < v1 ? v0 : v1, hi = v0 < v1 ? v1 : v0;
-        v0 = lo;
-        v1 = hi;
-      } else {
-        const bool lower = (lane & j) == 0;
-        const unsigned long long o0 = __shfl_xor_sync(0xffffffffu, v0, j);
-        const unsigned long long o1 = __shfl_xor_sync(0xffffffffu, v1, j);
-        const bool up0 = (lane & k) == 0, up1 = ((lane + 32) & k) == 0;
-        v0 = (lower == up0) ? (v0 < o0 ? v0 : o0) : (v0 < o0 ? o0 : v0);
-        v1 = (lower == up1) ? (v1 < o1 ? v1 : o1) : (v1 < o1 ? o1 : v1);
-      }
-    }
+// How many of v[0 .. n) are smaller than v[i], for i = tid / parts of the block:
+// `parts` (a power of two up to 32) neighbouring lanes share the count.  The
+// values are distinct.  Every thread of the block calls it.
+__device__ __forceinline__ int count_smaller(const unsigned long long* v, int n, int i, int parts) {
+  int cnt = 0;
+  if (i < n) {
+    const unsigned long long mine = v[i];
+    for (int j = threadIdx.x & (parts - 1); j < n; j += parts) cnt += v[j] < mine;
   }
+  for (int o = 1; o < parts; o <<= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
+  return cnt;
+}
+
+// Ascending sort of n (a power of two) values in shared memory by the block's
+// first n threads, one each: bitonic, partners within a warp by shuffles, others
+// through shared memory (10 exchanges for 512 values instead of 45).
+__device__ __forceinline__ void sort_one_each(unsigned long long* v, int n) {
+  const int i = threadIdx.x;
+  unsigned long long x = i < n ? v[i] : ~0ull;
+  for (int k = 2; k <= n; k <<= 1)
+    for (int j = k >> 1; j > 0; j >>= 1) {
+      unsigned long long y;
+      if (j < 32) {
+        y = __shfl_xor_sync(0xffffffffu, x, j);
+      } else {
+        __syncthreads();
+        if (i < n) v[i] = x;
+        __syncthreads();
+        y = i < n ? v[i ^ j] : ~0ull;
+      }
+      const bool small = ((i & j) == 0) == ((i & k) == 0);
+      x = small == (x < y) ? x : y;
+    }
+  __syncthreads();
+  if (i < n) v[i] = x;
+  __syncthreads();
 }
 
 // Selection modes: kSelAll takes the B costs to the elites, weights and u*;
@@ -86,7 +108,8 @@ __device__ __forceinline__ void select_body(const SelectArgs& a, unsigned char* 
   const int Bp = (B + 1) & ~1;
   uint32_t* keys = reinterpret_cast<uint32_t*>(sm_raw);
   unsigned long long* sel = reinterpret_cast<unsigned long long*>(keys + Bp);
-  __shared__ uint32_t hist[512];
+  __shared__ __align__(16) uint32_t hist[512];
+  __shared__ unsigned long long few[kFewElites];  // the elites in order, when there are few
   __shared__ uint32_t warp_tot[32];
   __shared__ uint32_t s_digit, s_below, s_lt, s_cnt, s_nb;
   __shared__ double s_red[32];
@@ -209,12 +232,9 @@ __device__ __forceinline__ void select_body(const SelectArgs& a, unsigned char* 
     __syncthreads();
     if (wid == 0) {
       // lane l owns digits 8l .. 8l+7
-      uint32_t c[8], sum = 0;
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        c[q] = cur[lane * 8 + q];
-        sum += c[q];
-      }
+      const uint4 c_lo = reinterpret_cast<const uint4*>(cur)[2 * lane], c_hi = reinterpret_cast<const uint4*>(cur)[2 * lane + 1];
+      const uint32_t c[8] = {c_lo.x, c_lo.y, c_lo.z, c_lo.w, c_hi.x, c_hi.y, c_hi.z, c_hi.w};
+      const uint32_t sum = c[0] + c[1] + c[2] + c[3] + c[4] + c[5] + c[6] + c[7];
       uint32_t incl = sum;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
@@ -242,11 +262,16 @@ __device__ __forceinline__ void select_body(const SelectArgs& a, unsigned char* 
     }
   }
   const int Ep = next_pow2(E);
+  int parts = 1;  // lanes per counted pair: the block's threads over up to 128 pairs
+  while (parts < 32 && 256 * parts <= (int)blockDim.x) parts <<= 1;
+  const int pair = tid / parts;
+  int n_sel = E;  // pairs in sel
   if (boundary) {
     // The bin holding the E-th key has at most kBoundaryMax keys: every key
-    // below the bin is an elite, and the bin's keys are sorted by
-    // (key, index) in one warp to take the `rank` still needed.
-    unsigned long long* bnd = sel + Ep;
+    // below the bin is an elite, and so are the `rank` smallest (key, index)
+    // pairs of the bin, which follow the others in sel.
+    const int lt = E - (int)rank;
+    unsigned long long* bnd = sel + lt;
     if (tid == 0) {
       s_lt = 0;
       s_nb = 0;
@@ -269,17 +294,19 @@ __device__ __forceinline__ void select_body(const SelectArgs& a, unsigned char* 
       }
     }
     __syncthreads();
-    if (wid == 0) {
-      const int nb = (int)s_nb;
-      unsigned long long v0 = lane < nb ? bnd[lane] : ~0ull;
-      unsigned long long v1 = lane + 32 < nb ? bnd[lane + 32] : ~0ull;
-      warp_sort64(v0, v1, lane);
-      const uint32_t base = (uint32_t)E - rank;  // == s_lt
-      if ((uint32_t)lane < rank) sel[base + lane] = v0;
-      if ((uint32_t)(lane + 32) < rank) sel[base + lane + 32] = v1;
+    const int nb = (int)s_nb;
+    if (E <= kFewElites) {
+      n_sel = lt + nb;  // ordered together below
+    } else {
+      // the bin's smallest to the places after the others
+      const int r = count_smaller(bnd, nb, pair, parts);
+      const unsigned long long mine = pair < nb ? bnd[pair] : 0ull;
+      __syncthreads();
+      if ((tid & (parts - 1)) == 0 && pair < nb && r < (int)rank) bnd[r] = mine;
+      __syncthreads();
+      for (int i = E + tid; i < Ep; i += blockDim.x) sel[i] = ~0ull;
+      __syncthreads();
     }
-    for (int i = E + tid; i < Ep; i += blockDim.x) sel[i] = ~0ull;
-    __syncthreads();
   } else {
   const uint32_t T = prefix;       // the E-th smallest key
   const uint32_t need_eq = rank;   // how many keys equal to T are taken
@@ -325,16 +352,18 @@ __device__ __forceinline__ void select_body(const SelectArgs& a, unsigned char* 
   __syncthreads();
   }
 
-  // bitonic sort of the E selected (key, index) pairs, ascending: in the
-  // registers of one warp for E <= 64, through shared memory otherwise
-  if (Ep <= 64) {
-    if (wid == 0) {
-      unsigned long long v0 = lane < Ep ? sel[lane] : ~0ull;
-      unsigned long long v1 = lane + 32 < Ep ? sel[lane + 32] : ~0ull;
-      warp_sort64(v0, v1, lane);
-      if (lane < Ep) sel[lane] = v0;
-      if (lane + 32 < Ep) sel[lane + 32] = v1;
-    }
+  // the E smallest of the selected (key, index) pairs in ascending order: of few,
+  // each takes the place that is its count of smaller ones (one barrier where
+  // two 21-stage sorts of one warp took 1.8 us); of many, a bitonic sort, one
+  // value per thread where the block has as many
+  unsigned long long* sorted = sel;
+  if (E <= kFewElites) {
+    sorted = few;
+    const int r = count_smaller(sel, n_sel, pair, parts);
+    if ((tid & (parts - 1)) == 0 && pair < n_sel && r < E) few[r] = sel[pair];
+    __syncthreads();
+  } else if (Ep <= (int)blockDim.x) {
+    sort_one_each(sel, Ep);
   } else {
     for (int k = 2; k <= Ep; k <<= 1) {
       for (int j = k >> 1; j > 0; j >>= 1) {
@@ -353,12 +382,11 @@ __device__ __forceinline__ void select_body(const SelectArgs& a, unsigned char* 
       }
     }
   }
-  __syncthreads();
 
   if constexpr (MODE == kSelChunk) {
     unsigned long long* out = a.pairs + (size_t)blockIdx.x * a.E;
     for (int k = tid; k < a.E; k += blockDim.x)
-      out[k] = k < E ? ((sel[k] & 0xffffffff00000000ull) | (unsigned long long)(uint32_t)(base + (int)(sel[k] & 0xffffffffu)))
+      out[k] = k < E ? ((sorted[k] & 0xffffffff00000000ull) | (unsigned long long)(uint32_t)(base + (int)(sorted[k] & 0xffffffffu)))
                      : ~0ull;
     return;
   }
@@ -370,48 +398,48 @@ __device__ __forceinline__ void select_body(const SelectArgs& a, unsigned char* 
   };
   // u* = U[elite[0], 0, :], requested before the softmax so the load
   // overlaps it
-  const int best_row = index_of_sel(sel[0]);
-  if (E <= 64) {
-    // One warp, elites lane and lane + 32, their costs decoded from the
-    // sorted order keys (no global reload), no block barrier.  The two
-    // halves are reduced separately and then added, which is the order of
-    // the block-wide reduction below for the same E, so the weights are the
-    // same bits either way.
-    if (wid != 0) return;
-    const float u_best = lane < a.n ? a.U[(size_t)best_row * a.H * a.n + lane] : 0.f;
-    const double best = (double)key_cost((uint32_t)(sel[0] >> 32));
+  const int best_row = index_of_sel(sorted[0]);
+  if (E <= kFewElites) {
+    // Warp h takes elites 32 h + lane, on FP64 pipes of their own (64 cycles an
+    // instruction: the exponentials of both halves on one pipe took 0.9 us more);
+    // their costs are decoded from the order keys (no global reload).  The two
+    // halves are reduced separately and then added, which is the order of the
+    // block-wide reduction below for the same E, so the weights are the same
+    // bits either way.
+    const int warps = E > 32 ? 2 : 1;
+    if (wid >= warps) return;
+    const float u_best = tid < a.n ? a.U[(size_t)best_row * a.H * a.n + tid] : 0.f;
+    const double best = (double)key_cost((uint32_t)(sorted[0] >> 32));
     const bool uniform = (a.update_rule == MTP_UPDATE_PLAIN_CEM) || !(best < INFINITY);
-    double w[2] = {0.0, 0.0};
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int k = lane + 32 * h;
-      if (k < E) {
-        const unsigned long long e = sel[k];
-        const int idx = index_of_sel(e);
-        a.elite[k] = idx;
-        if (a.elite_out) a.elite_out[k] = idx;
-        const double c = (double)key_cost((uint32_t)(e >> 32));
-        w[h] = uniform ? 1.0 : exp(-(c - best) * a.inv_lambda);
-      }
+    double w = 0.0;
+    if (tid < E) {
+      const unsigned long long e = sorted[tid];
+      const int idx = index_of_sel(e);
+      a.elite[tid] = idx;
+      if (a.elite_out) a.elite_out[tid] = idx;
+      const double c = (double)key_cost((uint32_t)(e >> 32));
+      w = uniform ? 1.0 : exp(-(c - best) * a.inv_lambda);
     }
-    double s0 = w[0], s1 = w[1];
+    double sum = w;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      s0 += __shfl_xor_sync(0xffffffffu, s0, o);
-      s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if (warps == 2) {
+      if (lane == 0) s_red[wid] = sum;
+      asm volatile("bar.sync 1, 64;" ::: "memory");  // the two warps
+      sum = s_red[0] + s_red[1];
     }
-    const double inv_total = 1.0 / (s0 + s1);
-    if (lane < E) a.weight[lane] = w[0] * inv_total;
-    if (lane + 32 < E) a.weight[lane + 32] = w[1] * inv_total;
-    if (lane < a.n) {
-      a.ustar[lane] = u_best;
-      if (a.ustar_out) a.ustar_out[lane] = u_best;
+    const double inv_total = 1.0 / sum;
+    if (tid < E) a.weight[tid] = w * inv_total;
+    if (tid < a.n) {
+      a.ustar[tid] = u_best;
+      if (a.ustar_out) a.ustar_out[tid] = u_best;
     }
     return;
   }
   const float u_best = tid < a.n ? a.U[(size_t)best_row * a.H * a.n + tid] : 0.f;
-  // softmax weights over the elites (FP64), shifted by the best cost
-  const double best = (double)a.cost[best_row];
+  // softmax weights over the elites (FP64), shifted by the best cost; the costs
+  // are decoded from the order keys
+  const double best = (double)key_cost((uint32_t)(sorted[0] >> 32));
   const bool uniform = (a.update_rule == MTP_UPDATE_PLAIN_CEM) || !(best < INFINITY);
   double part = 0.0;
   // elites on consecutive threads: the FP64 pipe is occupied per warp
@@ -422,11 +450,10 @@ __device__ __forceinline__ void select_body(const SelectArgs& a, unsigned char* 
   const int k0 = tid;
   double w_first = 0.0;
   for (int k = k0; k < E; k += blockDim.x) {
-    const int idx = index_of_sel(sel[k]);
+    const int idx = index_of_sel(sorted[k]);
     a.elite[k] = idx;
     if (a.elite_out) a.elite_out[k] = idx;
-    double c = (double)a.cost[idx];
-    if (isnan(c)) c = INFINITY;
+    const double c = (double)key_cost((uint32_t)(sorted[k] >> 32));
     const double w = uniform ? 1.0 : exp(-(c - best) * a.inv_lambda);
     if (k == k0) w_first = w;
     else a.weight[k] = w;
@@ -508,35 +535,48 @@ constexpr int kUpdRounds = 2;
 // Threads per block of the update launches.
 constexpr int kUpdThreads = 128;
 
+// The same for more than 64 elites: a pass then waits for two loads (from device
+// memory: the elites' rows) per eight rounds (65536 candidates, 512 elites: the
+// update 17 -> 15.5 us under ncu).
+constexpr int kUpdRoundsMany = 8;
+
 // The new mean and spread of element e from the sums over the elites of
 // d = u - c and w d^2 (shift c), then the floor and the smoothing.
-__device__ __forceinline__ void finish_element(const UpdateArgs& a, int e, double c, double S1,
-                                               double S2, bool cem) {
+__device__ __forceinline__ void finish_mean(const UpdateArgs& a, int e, double c, double S1, bool cem) {
+  double mn;
   if (cem) {
     // Sec. 2.1 CEM update: mean and unbiased variance of the elites
     const double E = (double)a.E;
     const double m1 = c + S1 / E;
-    const double ss = fmax(S2 - S1 * (S1 / E), 0.0);
-    const double s1 = a.E > 1 ? sqrt(ss / (E - 1.0)) : 0.0;
-    const double mn = a.alpha * a.mu[e] + (1.0 - a.alpha) * m1;
-    const double sn = a.alpha * a.sigma[e] + (1.0 - a.alpha) * s1;
-    a.mu[e] = mn;
-    a.sigma[e] = sn;
-    a.mu_f[e] = (float)mn;
-    a.sigma_f[e] = (float)sn;
+    mn = a.alpha * a.mu[e] + (1.0 - a.alpha) * m1;
   } else {
     // Alg. 2: weighted mean and standard deviation (weights sum to one)
     const double m1 = c + S1;
+    mn = m1 + a.alpha * (a.mu[e] - m1);
+  }
+  a.mu[e] = mn;
+  a.mu_f[e] = (float)mn;
+}
+__device__ __forceinline__ void finish_spread(const UpdateArgs& a, int e, double S1, double S2, bool cem) {
+  double sn;
+  if (cem) {
+    const double E = (double)a.E;
+    const double ss = fmax(S2 - S1 * (S1 / E), 0.0);
+    const double s1 = a.E > 1 ? sqrt(ss / (E - 1.0)) : 0.0;
+    sn = a.alpha * a.sigma[e] + (1.0 - a.alpha) * s1;
+  } else {
     double s1 = sqrt(fmax(S2 - S1 * S1, 0.0));
     if (s1 < a.sigma_min) s1 = a.sigma_min;
-    const double mn = m1 + a.alpha * (a.mu[e] - m1);
-    const double sn = s1 + a.alpha * (a.sigma[e] - s1);
-    a.mu[e] = mn;
-    a.sigma[e] = sn;
-    a.mu_f[e] = (float)mn;
-    a.sigma_f[e] = (float)sn;
+    sn = s1 + a.alpha * (a.sigma[e] - s1);
   }
+  a.sigma[e] = sn;
+  a.sigma_f[e] = (float)sn;
 }
+
+template <int V>
+struct Rounds {
+  static constexpr int value = V;
+};
 
 // Groups of G lanes each own one (t, i) element.  Thread `gt` of `threads`
 // threads given to one planning problem.
@@ -550,9 +590,10 @@ __device__ __forceinline__ void update_body(const UpdateArgs& a, int gt, int thr
   // G > 1: the loop runs block-uniformly (as many sweeps as the block's first
   // group needs; groups past the end idle through the shuffles), so that
   // each sweep ends with the block's elements finished together: lane 0 of
-  // each group leaves its sums in shared memory and thread s finishes group
-  // s's element.  That is one stream of FP64 instructions for all of the
-  // block's elements instead of one per element, with the same arithmetic.
+  // each group leaves its sums in shared memory and two threads finish its
+  // element, one its mean and one its spread.  That is two streams of FP64
+  // instructions for all of the block's elements instead of one per element,
+  // with the same arithmetic.
   const int per_sweep = (G == 1) ? threads : (threads / 32) * (32 / G);
   const int first = (G == 1) ? gt : (gt / 32) * (32 / G) + (threadIdx.x & 31) / G;
   const int block_first = ((gt - (int)threadIdx.x) / 32) * (32 / G);
@@ -578,41 +619,48 @@ __device__ __forceinline__ void update_body(const UpdateArgs& a, int gt, int thr
     // weights, so a pass over the elites waits for two dependent loads
     // rather than two per round.  With many, the P gathers of one round are
     // already independent and issued together (R = 1).
+    auto rounds = [&](auto RR) {
+      constexpr int R = decltype(RR)::value;
+      for (int k0 = 0; k0 < a.E; k0 += 32 * R) {
+        int idx[R][P];
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+          for (int j = 0; j < P; ++j) {
+            const int k = k0 + 32 * r + sub + G * j;
+            idx[r][j] = k < a.E ? __ldg(a.elite + k) : 0;
+          }
+        float uv[R][P];
+        double wv[R][P];
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+          for (int j = 0; j < P; ++j) {
+            const int k = k0 + 32 * r + sub + G * j;
+            uv[r][j] = k < a.E ? __ldg(a.U + (size_t)idx[r][j] * Hn + e) : 0.f;
+            wv[r][j] = (k < a.E && !cem) ? a.weight[k] : 1.0;
+          }
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+          for (int j = 0; j < P; ++j) {
+            const int k = k0 + 32 * r + sub + G * j;
+            if (k < a.E) {
+              const double d = (double)uv[r][j] - c;
+              const double wd = cem ? d : wv[r][j] * d;
+              p1[j] = p1[j] + wd;
+              p2[j] = fma(wd, d, p2[j]);
+            }
+          }
+      }
+    };
     constexpr int R = P == 1 ? kUpdRounds : (P == 2 ? kUpdRounds / 2 : 1);
     if (valid) {
-      if constexpr (R > 1) {
-        for (int k0 = 0; k0 < a.E; k0 += 32 * R) {
-          int idx[R][P];
-#pragma unroll
-          for (int r = 0; r < R; ++r)
-#pragma unroll
-            for (int j = 0; j < P; ++j) {
-              const int k = k0 + 32 * r + sub + G * j;
-              idx[r][j] = k < a.E ? __ldg(a.elite + k) : 0;
-            }
-          float uv[R][P];
-          double wv[R][P];
-#pragma unroll
-          for (int r = 0; r < R; ++r)
-#pragma unroll
-            for (int j = 0; j < P; ++j) {
-              const int k = k0 + 32 * r + sub + G * j;
-              uv[r][j] = k < a.E ? __ldg(a.U + (size_t)idx[r][j] * Hn + e) : 0.f;
-              wv[r][j] = (k < a.E && !cem) ? a.weight[k] : 1.0;
-            }
-#pragma unroll
-          for (int r = 0; r < R; ++r)
-#pragma unroll
-            for (int j = 0; j < P; ++j) {
-              const int k = k0 + 32 * r + sub + G * j;
-              if (k < a.E) {
-                const double d = (double)uv[r][j] - c;
-                const double wd = cem ? d : wv[r][j] * d;
-                p1[j] = p1[j] + wd;
-                p2[j] = fma(wd, d, p2[j]);
-              }
-            }
-        }
+      if constexpr (P == 1) {
+        if (a.E > 64) rounds(Rounds<kUpdRoundsMany>{});
+        else rounds(Rounds<R>{});
+      } else if constexpr (R > 1) {
+        rounds(Rounds<R>{});
       } else {
         for (int k0 = 0; k0 < a.E; k0 += 32) {
 #pragma unroll
@@ -631,7 +679,10 @@ __device__ __forceinline__ void update_body(const UpdateArgs& a, int gt, int thr
     const double S1 = canonical_sum<G>(p1);
     const double S2 = canonical_sum<G>(p2);
     if constexpr (G == 1) {
-      if (valid) finish_element(a, e, c, S1, S2, cem);
+      if (valid) {
+        finish_mean(a, e, c, S1, cem);
+        finish_spread(a, e, S1, S2, cem);
+      }
     } else {
       const int slot = threadIdx.x / G;
       if (sub == 0) {
@@ -641,8 +692,14 @@ __device__ __forceinline__ void update_body(const UpdateArgs& a, int gt, int thr
         sh_e[slot] = valid ? e : -1;
       }
       __syncthreads();
-      if (threadIdx.x < kGroups && sh_e[threadIdx.x] >= 0)
-        finish_element(a, sh_e[threadIdx.x], sh_c[threadIdx.x], sh_S1[threadIdx.x], sh_S2[threadIdx.x], cem);
+      // the spreads on the block's first threads, the means on its second half:
+      // FP64 pipes of their own
+      static_assert(kGroups <= kUpdThreads / 2, "both fit the block");
+      const int z = threadIdx.x & (kUpdThreads / 2 - 1);
+      if (z < kGroups && sh_e[z] >= 0) {
+        if (threadIdx.x < kUpdThreads / 2) finish_spread(a, sh_e[z], sh_S1[z], sh_S2[z], cem);
+        else finish_mean(a, sh_e[z], sh_c[z], sh_S1[z], cem);
+      }
       __syncthreads();  // the next sweep rewrites the slots
     }
   }
@@ -794,7 +851,7 @@ constexpr int kSelKeys = 4;
 
 int select_threads(int B, int E) {
   int t = (B + kSelKeys - 1) / kSelKeys;
-  if (t < E) t = E;
+  if (t < E) t = next_pow2(E);
   t = (t + 31) & ~31;
   if (t < 128) t = 128;
   if (t > kSelThreads) t = kSelThreads;
@@ -815,7 +872,10 @@ void select_plan(int B, int E, int* chunk, int* chunks) {
   *chunk = B;
   *chunks = 0;
   if (select_smem_bytes(B, E) <= kSelSmemMax && B <= kOneBlockMax) return;
-  int c = kChunkKeys;
+  // shorter chunks put more blocks to work, as long as their pairs stay few
+  // (65536 costs, 512 elites: 4 chunks of 16384 took 19 + 14.5 us)
+  int c = kChunkLeast;
+  while (c < kChunkKeys && ((long long)B + c - 1) / c * E > 8192) c <<= 1;
   while (c > E && select_smem_bytes(c, E) > kSelSmemMax) c >>= 1;
   if (c < E) c = E;
   const long long n = ((long long)B + c - 1) / c;

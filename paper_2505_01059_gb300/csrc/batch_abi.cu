@@ -55,8 +55,6 @@ constexpr int kMaxGroups = 64;
 #endif
 constexpr double kPersistSplitFraction = MTP_PERSIST_SPLIT_FRACTION;
 constexpr int kPersistFirstFewer = MTP_PERSIST_FIRST_FEWER;
-// Horizon chunk of staged control loads before the autotuner has run.
-constexpr int kDefaultChunk = 4;
 constexpr size_t kBatchGraphSmem = 40 * 1024;  // four graph blocks per SM
 // Groups of four elements per thread of the local rows, each thread on one q
 // group of several rows, so that its set-up (instance search, box, the group's
@@ -306,7 +304,7 @@ cudaError_t fill_batch(mtp_batch* b, mtp_handle* const* handles, int count, cuda
       g.model_first = n_dyn[dyn];
       auto it = b->tuned.find({dyn, n});
       g.block = it != b->tuned.end() ? it->second[0] : 128;
-      g.chunk = it != b->tuned.end() ? it->second[1] : kDefaultChunk;
+      g.chunk = it != b->tuned.end() ? it->second[1] : chain_chunk(n);  // before tuning: staged
       b->groups.push_back(g);
     }
     ++b->groups.back().count;
@@ -975,17 +973,16 @@ mtp_status mtp_batch_autotune(mtp_batch* b, int32_t* tiles_out, int32_t* n_group
   // rollout tiles: threads per block (the kernels are bounded at 128) x, for
   // chains, the horizon chunk of the staged control loads (0: direct loads)
   const int blocks[3] = {32, 64, 128};
-  const int chunks[2] = {0, 4};
   cudaEvent_t t0, t1;
   cudaEventCreate(&t0);
   cudaEventCreate(&t1);
   cudaError_t e = cudaSuccess;
   struct Tile {
-    int block, chunk;
+    int block, chunk;  // chunk: staged or not, then the group's chunk length
   };
   std::vector<Tile> tiles;
-  for (int chunk : chunks)
-    for (int block : blocks) tiles.push_back({block, chunk});
+  for (int staged = 0; staged < 2; ++staged)
+    for (int block : blocks) tiles.push_back({block, staged});
   auto group_steps = [&](const BatchGroup& g) {
     long long steps = 0;
     for (int j = 0; j < g.count; ++j) steps += (long long)b->hs_sorted[g.first + j]->dm.B * b->hs_sorted[g.first + j]->dm.H;
@@ -994,7 +991,8 @@ mtp_status mtp_batch_autotune(mtp_batch* b, int32_t* tiles_out, int32_t* n_group
   for (auto& g : b->groups) {
     float best = 1e30f;
     Tile best_tile{g.block, g.chunk};
-    for (const Tile& tl : tiles) {
+    for (Tile tl : tiles) {
+      if (tl.chunk) tl.chunk = chain_chunk(g.n);
       // the legged rollout has one fixed tile: timed once, for the launch order
       if (g.dyn == MTP_DYN_LEGGED && (tl.block != blocks[0] || tl.chunk)) continue;
       if (tl.chunk && !g.stageable) continue;

@@ -317,7 +317,6 @@ RolloutArgs rollout_args(const mtp_handle* h, uint32_t iter, const uint32_t* d_i
   a.rows = rows;
   a.cost = cost;
   a.kahan = (h->pr.flags & MTP_FLAG_NO_KAHAN) ? 0 : 1;
-  a.status = h->status;
   return a;
 }
 
@@ -1179,7 +1178,7 @@ mtp_status mtp_device_status(mtp_handle* h) {
   if (word == 0) return MTP_OK;
   MTP_CUDA(h, cudaMemset(h->status, 0, 4));
   return fail(h, MTP_ERR_TIMEOUT,
-              "a rollout's bounded wait for its staged controls gave up (those candidates cost +inf)");
+              "the tensor-core contraction's bounded wait gave up (those graph rows were not written)");
 }
 
 mtp_status mtp_get_state(mtp_handle* h, double* h_mu, double* h_sigma, uint32_t* h_iter) {

@@ -194,18 +194,18 @@ struct RolloutArgs {
   float* cost;       // (rows)
   float* X;          // (H+1, d) states of the single requested row, or null
   int32_t kahan;
-  uint32_t* status;  // device status word of the handle (bits set by a rollout), or null
 };
 
-// Bits of a handle's device status word, set when a bounded wait gave up:
-// a rollout's wait for its staged controls (those candidates cost +inf), or
-// the tensor-core contraction's wait for its MMA (those graph rows are not
-// written).
-constexpr uint32_t kStatusStageTimeout = 1u;
+// Bit of a handle's device status word, set when a bounded wait gave up: the
+// tensor-core contraction's wait for its MMA (those graph rows are not written).
 constexpr uint32_t kStatusTcTimeout = 2u;
 
+// Steps per chunk of a chain's staged controls: 8 where two chunks of 32 rows
+// take 17 KB (what lets three persistent CTAs share an SM), else 4.
+__host__ __device__ constexpr int chain_chunk(int links) { return links <= 8 ? 8 : 4; }
+
 // Whether a rollout launch may stage its controls through shared memory with
-// bulk copies (see StagedRows): 16-byte aligned rows of a multiple of 4
+// 16-byte copies (see StagedRows): 16-byte aligned rows of a multiple of 4
 // floats, one model per candidate, no state output.
 inline bool can_stage(const RolloutArgs& a, int k) {
   return a.X == nullptr && a.dr_mode != MTP_DR_SHARED &&
@@ -282,8 +282,8 @@ cudaError_t launch_candidates(const CandArgs& a, int local_blocks, cudaStream_t 
 cudaError_t launch_sample_tensor(const Dims& dm, Key key, uint32_t iter, const float* umin,
                                  const float* umax, float* Z, int32_t* I, float* C,
                                  cudaStream_t s);
-// Rollouts: `chunk` is the horizon chunk of staged control loads (4 or 8
-// steps; 0, or a launch that cannot stage, loads directly).
+// Rollouts: with `chunk` a chain's controls are staged chain_chunk steps at a
+// time (0, or a launch that cannot stage, loads directly).
 cudaError_t init_rollout_pm_attributes();
 cudaError_t init_rollout_chain_attributes();
 cudaError_t init_rollout_pm_batch_attributes();
@@ -317,7 +317,7 @@ struct PersistArgs {
   unsigned* head;     // the tile counter, zeroed by the launch
   int count, total_warps;
   int w_base;         // wstart[0]: the first tile of these entries in the batch's numbering
-  size_t warp_bytes;  // shared memory per warp: two mbarriers and the largest tile
+  size_t warp_bytes;  // shared memory per warp: the largest tile
   int staged;         // chain tiles stage their controls where their rows allow it (else direct loads)
 };
 // Shared memory per warp: a point mass's tile of `axes` axes, in floats; and

@@ -1,7 +1,5 @@
 // rollout_chain.cu -- launcher of the standalone planar-chain rollout, with
-// direct or staged control loads (rollout_kernels.cuh).  Chains stage 4
-// steps at a time: their long step bodies need no longer chunks to hide the
-// copies.
+// direct or staged control loads (rollout_kernels.cuh).
 #include "rollout_kernels.cuh"
 
 namespace mtp {
@@ -20,7 +18,7 @@ template <int NL>
 cudaError_t chain_dispatch(const RolloutArgs& a, const ChainModel& m, int links, int chunk,
                            cudaStream_t s) {
   if constexpr (NL <= kMaxChainLinks) {
-    if (links == NL) return chunk ? chain_launch<NL, 4>(a, m, s) : chain_launch<NL, 0>(a, m, s);
+    if (links == NL) return chunk ? chain_launch<NL, chain_chunk(NL)>(a, m, s) : chain_launch<NL, 0>(a, m, s);
     return chain_dispatch<NL + 1>(a, m, links, chunk, s);
   } else {
     return cudaErrorInvalidValue;
@@ -30,8 +28,8 @@ cudaError_t chain_dispatch(const RolloutArgs& a, const ChainModel& m, int links,
 template <int NL>
 cudaError_t chain_attributes() {
   if constexpr (NL <= kMaxChainLinks) {
-    cudaError_t e = cudaFuncSetAttribute(k_rollout_chain<NL, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)staged_smem<NL, 4>(kThreads));
+    cudaError_t e = cudaFuncSetAttribute(k_rollout_chain<NL, chain_chunk(NL)>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)staged_smem<NL, chain_chunk(NL)>(kThreads));
     if (e != cudaSuccess) return e;
     return chain_attributes<NL + 1>();
   } else {

@@ -1,6 +1,6 @@
 // rollout_chain_batch.cu -- launcher of the batched planar-chain rollout (one
 // launch over many instances of one link count), with direct or staged
-// control loads (rollout_kernels.cuh; chains stage 4 steps at a time).
+// control loads (rollout_kernels.cuh).
 #include "rollout_kernels.cuh"
 
 namespace mtp {
@@ -22,7 +22,7 @@ cudaError_t chain_batch_dispatch(const RolloutArgs* ra, const ChainModel* cm, co
                                  cudaStream_t s) {
   if constexpr (NL <= kMaxChainLinks) {
     if (links == NL)
-      return chunk ? chain_batch_launch<NL, 4>(ra, cm, row_start, count, total_rows, block, s)
+      return chunk ? chain_batch_launch<NL, chain_chunk(NL)>(ra, cm, row_start, count, total_rows, block, s)
                    : chain_batch_launch<NL, 0>(ra, cm, row_start, count, total_rows, block, s);
     return chain_batch_dispatch<NL + 1>(ra, cm, row_start, count, total_rows, links, block, chunk, s);
   } else {
@@ -33,9 +33,9 @@ cudaError_t chain_batch_dispatch(const RolloutArgs* ra, const ChainModel* cm, co
 template <int NL>
 cudaError_t chain_batch_attributes() {
   if constexpr (NL <= kMaxChainLinks) {
-    cudaError_t e = cudaFuncSetAttribute(k_rollout_chain_batch<NL, 4>,
+    cudaError_t e = cudaFuncSetAttribute(k_rollout_chain_batch<NL, chain_chunk(NL)>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)staged_smem<NL, 4>(kThreads));
+                                         (int)staged_smem<NL, chain_chunk(NL)>(kThreads));
     if (e != cudaSuccess) return e;
     return chain_batch_attributes<NL + 1>();
   } else {

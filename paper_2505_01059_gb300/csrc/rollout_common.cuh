@@ -74,35 +74,6 @@ __device__ __forceinline__ void copy_async_f32(float* smem_dst, const float* gme
 __device__ __forceinline__ void copy_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void copy_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
-// ---------------------------------------------------------------------------
-// Staged control rows.  A rollout thread reads its candidate's controls one
-// step after another; a warp's 32 lanes read 32 different rows, H * n floats
-// apart, so each direct warp load touches 32 cache lines (measured: 31
-// sectors per request and the L1 at 83-93 % of its throughput in the batched
-// 7-link and 9-axis rollouts, whose issue slots were 44 % and 22 % busy).
-// Staged instead, each warp's rows pass through shared memory a horizon
-// chunk of T steps at a time: lane l issues one bulk copy (cp.async.bulk,
-// the TMA engine's untiled form) of row l's next T * K floats, an mbarrier
-// per buffer counts the bytes, and two buffers alternate so that chunk c + 1
-// arrives while chunk c is used.  A bulk copy needs 16-byte aligned source,
-// destination and size: the host stages only rows whose base is 16-byte
-// aligned and whose length H * K is a multiple of 4 floats, with T a
-// multiple of 4, so every chunk start and length is a multiple of 16 bytes.
-// The row stride in shared memory is a multiple of 4 floats with an odd
-// quotient, so that the lanes' 16-byte row starts fall in distinct bank
-// quads (a scalar read is then a 4-way conflict, against 32 lines per direct
-// warp load).
-// ---------------------------------------------------------------------------
-template <int K, int T>
-struct StageShape {
-  static_assert(T % 4 == 0, "chunks must be whole 16-byte units");
-  static constexpr int kRow = T * K;
-  static constexpr int kQuads = (kRow + 3) / 4;
-  static constexpr int kStride = 4 * (kQuads % 2 ? kQuads : kQuads + 1);  // floats
-  static constexpr int kBuf = 32 * kStride;                                 // floats per buffer
-  static constexpr size_t kWarpBytes = 2 * kBuf * sizeof(float) + 16;       // + two mbarriers
-};
-
 // Bounded mbarrier wait: try_wait on the phase with the given parity for at
 // most limit_ns of the global timer (about two seconds by default), then
 // give up (returns false).
@@ -127,121 +98,101 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
   }
 }
 
-// The two mbarriers of a warp's staging, initialised by one lane.
-__device__ __forceinline__ void init_stage_bars(uint64_t* bars) {
-  if ((threadIdx.x & 31) == 0) {
-    const unsigned b0 = (unsigned)__cvta_generic_to_shared(bars);
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(b0) : "memory");
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(b0 + 8) : "memory");
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  __syncwarp();
+// ---------------------------------------------------------------------------
+// Staged control rows.  A rollout thread reads its candidate's controls one
+// step after another; a warp's 32 lanes read 32 different rows, H * n floats
+// apart, so each direct warp load touches 32 cache lines (measured: 31
+// sectors per request and the L1 at 83-93 % of its throughput in the batched
+// 7-link and 9-axis rollouts).  Staged instead, the rows pass through shared
+// memory a horizon chunk of T steps at a time: the warp copies the next chunk of
+// all its rows with asynchronous 16-byte copies, neighbouring lanes on
+// neighbouring pieces, into the one of two buffers that it does not read.  The
+// host stages only rows whose base is 16-byte aligned and whose length H * K is
+// a multiple of 4 floats, with T a multiple of 4, so every chunk is whole
+// pieces.  (One bulk copy per lane and an mbarrier per buffer, as before, took
+// about 300 instructions of the integer pipe per chunk in the protocol and its
+// bounded wait.)  The row stride in shared memory is a multiple of 4 floats with
+// an odd quotient, so that the lanes' 16-byte row starts fall in distinct bank
+// quads (a scalar read is then a 4-way conflict, against 32 lines per direct
+// warp load).
+// ---------------------------------------------------------------------------
+template <int K, int T>
+struct StageShape {
+  static_assert(T % 4 == 0, "chunks must be whole 16-byte units");
+  static constexpr int kQuads = (T * K + 3) / 4;
+  static constexpr int kStride = 4 * (kQuads % 2 ? kQuads : kQuads + 1);  // floats
+  static constexpr int kBuf = 32 * kStride;                               // floats per buffer
+  static constexpr size_t kWarpBytes = 2 * kBuf * sizeof(float);
+};
+
+__device__ __forceinline__ void copy_async_16(float* smem_dst, const float* gmem_src) {
+  const unsigned dst = (unsigned)__cvta_generic_to_shared(smem_dst);
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(gmem_src) : "memory");
 }
 
+// Asynchronous copies, by one warp, of n candidates' next `steps` steps of
+// controls (src, H K floats apart) into rows `row` floats apart: in 16-byte
+// pieces (vec: every piece is aligned) or by single floats.
+template <int K>
+__device__ __forceinline__ void copy_controls(const float* src, int H, int n, int steps, bool vec, float* dst, int row) {
+  const int lane = threadIdx.x & 31;
+  const int len = vec ? steps * K / 4 : steps * K;  // pieces per candidate
+  int i = lane / len, o = lane - i * len;
+  const int di = 32 / len, dlen = 32 - di * len;
+  while (i < n) {
+    if (vec) copy_async_16(dst + i * row + 4 * o, src + (size_t)i * H * K + 4 * o);
+    else copy_async_f32(dst + i * row + o, src + (size_t)i * H * K + o);
+    i += di;
+    o += dlen;
+    if (o >= len) {
+      o -= len;
+      ++i;
+    }
+  }
+  copy_async_commit();
+}
+
+// The rows of a warp's candidates (the first one's, and how many there are) and
+// its two buffers.
 template <int K, int T>
 struct StagedRows {
   using Shape = StageShape<K, T>;
-  float* buf;        // [2][32][kStride]
-  uint64_t* bar;     // [2]
-  const float* row;  // this lane's row (null when the lane has no candidate)
-  int H, chunks;
-  int seq;           // chunks consumed so far (buffer and phase of the next one)
-  uint32_t live;     // lanes with a candidate
-  int lane;
-
-  // `smem` is this warp's kWarpBytes of shared memory (16-byte aligned).
-  // Every lane of the warp calls it.
-  __device__ __forceinline__ void init(unsigned char* smem, const float* my_row, int H_) {
-    buf = reinterpret_cast<float*>(smem);
-    bar = reinterpret_cast<uint64_t*>(smem + 2 * Shape::kBuf * sizeof(float));
-    row = my_row;
-    H = H_;
-    chunks = (H + T - 1) / T;
-    seq = 0;
-    lane = threadIdx.x & 31;
-    live = __ballot_sync(0xffffffffu, my_row != nullptr);
-    if (lane == 0) {
-      const unsigned b0 = (unsigned)__cvta_generic_to_shared(bar);
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(b0) : "memory");
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(b0 + 8) : "memory");
-      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  const float* rows;
+  int n;
+  float* buf;
+  // steps t0 .. t0 + T - 1 (those below H) into buffer b; every lane calls it
+  __device__ __forceinline__ void request(int t0, int H, int b) const {
+    const int lane = threadIdx.x & 31;
+    float* const dst = buf + b * Shape::kBuf;
+    const float* const src = rows + (size_t)t0 * K;
+    if (t0 + T <= H) {
+      // a whole chunk: T K / 4 pieces per lane, their rows known but for the
+      // lane's first
+      constexpr int len = T * K / 4, di = 32 / len, dlen = 32 - di * len;
+      int i = lane / len, o = lane - i * len;
+#pragma unroll 1
+      for (int q = 0; q < len; ++q) {
+        if (i < n) copy_async_16(dst + i * Shape::kStride + 4 * o, src + (size_t)i * H * K + 4 * o);
+        i += di;
+        o += dlen;
+        if (o >= len) {
+          o -= len;
+          ++i;
+        }
+      }
+      copy_async_commit();
+    } else {
+      copy_controls<K>(src, H, n, H - t0, true, dst, Shape::kStride);
     }
-    __syncwarp();
-  }
-
-  // Binds this warp's next row set to barriers and buffers that the warp
-  // keeps across rows of different widths: `bars` holds two mbarriers
-  // initialised once (init_bars), `buffer` two buffers of at least kBuf
-  // floats, and `seq_` counts the chunks this warp has consumed on those
-  // barriers so far (it sets their phases).  Every lane calls it.
-  __device__ __forceinline__ void attach(uint64_t* bars, float* buffer, const float* my_row, int H_,
-                                         int seq_) {
-    buf = buffer;
-    bar = bars;
-    row = my_row;
-    H = H_;
-    chunks = (H + T - 1) / T;
-    seq = seq_;
-    lane = threadIdx.x & 31;
-    live = __ballot_sync(0xffffffffu, my_row != nullptr);
-  }
-
-  // Data chunk c (steps c*T ..) as the g-th chunk of this warp's sequence,
-  // into buffer g & 1.  Every lane of the warp calls it; the lanes' reads of
-  // that buffer's previous chunk have been consumed by then.
-  __device__ __forceinline__ void issue(int c, int g) {
-    __syncwarp();
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    const int t0 = c * T;
-    const int steps = min(T, H - t0);
-    const uint32_t bytes = (uint32_t)(steps * K * sizeof(float));
-    const unsigned b = (unsigned)__cvta_generic_to_shared(bar + (g & 1));
-    if (lane == 0) {
-      const uint32_t total = bytes * (uint32_t)__popc(live);
-      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(b), "r"(total)
-                   : "memory");
-    }
-    __syncwarp();
-    if (row) {
-      const unsigned dst = (unsigned)__cvta_generic_to_shared(buf + (g & 1) * Shape::kBuf +
-                                                              lane * Shape::kStride);
-      asm volatile(
-          "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-          ::"r"(dst), "l"(row + (size_t)t0 * K), "r"(bytes), "r"(b)
-          : "memory");
-    }
-  }
-
-  // Waits for the g-th chunk (bounded); false, on every lane, when the wait
-  // gave up.
-  __device__ __forceinline__ bool wait(int g) {
-    const bool ok = mbar_wait_bounded(bar + (g & 1), (uint32_t)((g >> 1) & 1));
-    return __all_sync(0xffffffffu, ok);
-  }
-
-  // This lane's floats of the g-th chunk.
-  __device__ __forceinline__ const float* chunk(int g) const {
-    return buf + (g & 1) * Shape::kBuf + lane * Shape::kStride;
-  }
-
-  // After a failed wait on the g-th chunk: waits (again bounded) for the
-  // copies still in flight into this warp's buffers (the g-th and, when it
-  // was issued, the next) before the warp may leave.
-  __device__ __forceinline__ void drain(int g, bool next_issued) {
-    mbar_wait_bounded(bar + (g & 1), (uint32_t)((g >> 1) & 1));
-    if (next_issued) mbar_wait_bounded(bar + ((g + 1) & 1), (uint32_t)(((g + 1) >> 1) & 1));
   }
 };
 
 // Feeds step(t, u) the K controls of every step t = 0 .. H-1 of this lane's
 // candidate row Ub.  T == 0: direct loads PF steps ahead into a rotating
 // register buffer (the loop is unrolled by PF so its slots are constants).
-// T > 0: the warp's rows staged through shared memory by `st` (initialised
-// by the caller on every lane of the warp).  Returns false when a staged wait
-// gave up; the remaining steps are then skipped.
+// T > 0: the warp's rows staged through shared memory (every lane calls it).
 template <int K, int PF, int T, class Step>
-__device__ __forceinline__ bool for_each_step(const float* Ub, int H, StagedRows<K, T>* st,
-                                              Step&& step) {
+__device__ __forceinline__ void for_each_step(const float* Ub, int H, const StagedRows<K, T>* st, Step&& step) {
   if constexpr (T == 0) {
     (void)st;
     float ubuf[PF][K];
@@ -265,33 +216,27 @@ __device__ __forceinline__ bool for_each_step(const float* Ub, int H, StagedRows
         }
       });
     }
-    return true;
   } else {
-    const int chunks = st->chunks;
-    const int g0 = st->seq;
-    st->issue(0, g0);
-    for (int c = 0; c < chunks; ++c) {
-      const bool next = c + 1 < chunks;
-      if (next) st->issue(c + 1, g0 + c + 1);
-      if (!st->wait(g0 + c)) {
-        st->drain(g0 + c, next);
-        st->seq = g0 + c + 1 + (next ? 1 : 0);
-        return false;
-      }
+    using Shape = StageShape<K, T>;
+    const float* const mine = st->buf + (threadIdx.x & 31) * Shape::kStride;
+    __syncwarp();  // the warp's previous rows have been used
+    st->request(0, H, 0);
+    for (int t0 = 0, b = 0; t0 < H; t0 += T, b ^= 1) {
+      copy_async_wait_all();
+      __syncwarp();  // this chunk is there, and the other buffer's has been used
+      if (t0 + T < H) st->request(t0 + T, H, b ^ 1);
       // a rolled loop over the chunk's steps: its reads need no constant
       // slots, and the step body stays one copy
-      const float* src = st->chunk(g0 + c);
-      const int steps = min(T, H - c * T);
+      const float* src = mine + b * Shape::kBuf;
+      const int t1 = min(t0 + T, H);
 #pragma unroll 1
-      for (int q = 0; q < steps; ++q) {
+      for (int t = t0; t < t1; ++t, src += K) {
         float u[K];
 #pragma unroll
-        for (int k = 0; k < K; ++k) u[k] = src[q * K + k];
-        step(c * T + q, u);
+        for (int k = 0; k < K; ++k) u[k] = src[k];
+        step(t, u);
       }
     }
-    st->seq = g0 + chunks;
-    return true;
   }
 }
 

@@ -8,8 +8,8 @@
 // final cost leaves the SM.  The loop bodies are fully unrolled over the
 // compile-time link count, so the per-step linear algebra lives in registers.
 // The controls reach a thread either by direct loads a few steps ahead (T = 0)
-// or staged through shared memory a horizon chunk of T = 4 steps at a time by
-// bulk copies (see StagedRows), picked per launch shape by the batch autotuner.
+// or staged through shared memory a horizon chunk of T steps at a time (see
+// StagedRows), picked per launch shape by the batch autotuner.
 //
 // Planar chain: the dynamics are evaluated in absolute link angles phi_j
 // (phi_j = q_1 + ... + q_j).  For uniform thin rods the Lagrangian gives the
@@ -54,13 +54,9 @@ constexpr size_t staged_smem(int block) {
 }
 
 // This warp's staging area in the block's dynamic shared memory.
-__device__ __forceinline__ unsigned char* warp_stage_area(size_t warp_bytes) {
+__device__ __forceinline__ float* warp_stage_area(size_t warp_bytes) {
   extern __shared__ __align__(16) unsigned char rollout_dyn_smem[];
-  return rollout_dyn_smem + (threadIdx.x >> 5) * warp_bytes;
-}
-
-__device__ __forceinline__ void report_stage_timeout(const RolloutArgs& a) {
-  if (a.status) atomicOr(a.status, kStatusStageTimeout);
+  return reinterpret_cast<float*>(rollout_dyn_smem + (threadIdx.x >> 5) * warp_bytes);
 }
 
 // ---------------------------------------------------------------------------
@@ -79,8 +75,8 @@ __device__ __forceinline__ void chain_tip(const float (&len)[NL], const float (&
 }
 
 template <int NL, int PF, int T>
-__device__ __forceinline__ bool rollout_chain_body(const RolloutArgs& a, const ChainModel& cm,
-                                                   int r, bool live, StagedRows<NL, T>* st) {
+__device__ __forceinline__ void rollout_chain_body(const RolloutArgs& a, const ChainModel& cm,
+                                                   int r, bool live, const StagedRows<NL, T>* st) {
   const int b = a.row0 + r;
   const uint32_t iter = a.d_iter ? *a.d_iter : a.iter;
   const float* Ub = a.U + (size_t)r * a.H * NL;
@@ -90,8 +86,7 @@ __device__ __forceinline__ bool rollout_chain_body(const RolloutArgs& a, const C
 #pragma unroll
   for (int j = 0; j < NL; ++j) len[j] = cm.length[j];
   float total = 0.f;
-  bool ok = true;
-  for (int mdl = 0; mdl < models && ok; ++mdl) {
+  for (int mdl = 0; mdl < models; ++mdl) {
     const uint32_t unit = (a.dr_mode == MTP_DR_SHARED) ? (uint32_t)mdl : (uint32_t)b;
     // Lagrangian constants: beta_j = m_j/2 + sum_{i>j} m_i, lb_j = l_j beta_j,
     // D_jj = l_j^2 (m_j/3 + sum_{i>j} m_i), G_j = g l_j beta_j.
@@ -130,7 +125,7 @@ __device__ __forceinline__ bool rollout_chain_body(const RolloutArgs& a, const C
       }
     }
     KahanSum J;
-    ok = for_each_step<NL, PF, T>(Ub, a.H, st, [&](int t, const float (&u)[NL]) {
+    for_each_step<NL, PF, T>(Ub, a.H, st, [&](int t, const float (&u)[NL]) {
       float c[NL], s[NL], tau[NL];
 #pragma unroll
       for (int j = 0; j < NL; ++j) {
@@ -307,12 +302,10 @@ __device__ __forceinline__ bool rollout_chain_body(const RolloutArgs& a, const C
     }
     total += J.s;
   }
-  if (!live) return ok;
+  if (!live) return;
   float cst = total / (float)models;
-  if (!isfinite(cst) || !ok) cst = __int_as_float(0x7f800000);
-  if (!ok) report_stage_timeout(a);
+  if (!isfinite(cst)) cst = __int_as_float(0x7f800000);
   a.cost[r] = cst;
-  return ok;
 }
 
 // Standalone launches: one thread per candidate row.  Direct loads (T = 0)
@@ -327,11 +320,10 @@ __global__ void __launch_bounds__(kThreads) k_rollout_chain(const RolloutArgs a,
     rollout_chain_body<NL, kPrefetchAlone, 0>(a, cm, r, true, nullptr);
   } else {
     if (__all_sync(0xffffffffu, r >= a.rows)) return;
-    const bool live = r < a.rows;
-    StagedRows<NL, T> st;
-    st.init(warp_stage_area(StageShape<NL, T>::kWarpBytes),
-            live ? a.U + (size_t)r * a.H * NL : nullptr, a.H);
-    rollout_chain_body<NL, kPrefetchAlone, T>(a, cm, r, live, &st);
+    const int r0 = r & ~31;
+    const StagedRows<NL, T> st{a.U + (size_t)r0 * a.H * NL, min(32, a.rows - r0),
+                               warp_stage_area(StageShape<NL, T>::kWarpBytes)};
+    rollout_chain_body<NL, kPrefetchAlone, T>(a, cm, r, r < a.rows, &st);
   }
 }
 
@@ -351,9 +343,9 @@ __global__ void __launch_bounds__(kThreads) k_rollout_chain_batch(const RolloutA
     if (!live) return;
     rollout_chain_body<NL, kPrefetchBatch, 0>(a, cm, r, true, nullptr);
   } else {
-    StagedRows<NL, T> st;
-    st.init(warp_stage_area(StageShape<NL, T>::kWarpBytes),
-            live ? a.U + (size_t)r * a.H * NL : nullptr, a.H);
+    const int r0 = r & ~31;  // rows are padded to whole warps
+    const StagedRows<NL, T> st{a.U + (size_t)r0 * a.H * NL, min(32, a.rows - r0),
+                               warp_stage_area(StageShape<NL, T>::kWarpBytes)};
     rollout_chain_body<NL, kPrefetchBatch, T>(a, cm, r, live, &st);
   }
 }

@@ -10,7 +10,7 @@
 // the launch repeatedly takes the next item from a device counter (one
 // atomic add per item), looks its instance up by binary search, and runs
 // that tile's rollout: a point mass of K axes, or a planar chain of L links with
-// direct control loads or staged 4 steps at a time.  A warp therefore
+// direct or staged control loads.  A warp therefore
 // moves between instances of different sizes and dynamics, while the warps
 // running at one time mostly run the same body.  The bodies are the
 // per-candidate rollouts of the other kernels (the same templates), so every
@@ -19,9 +19,7 @@
 // entries (w_base numbers the second range's tiles).
 //
 // The warps never wait on one another: an item, once taken, depends only on
-// the candidates generated before the launch.  A staged tile's waits are the
-// bounded waits of StagedRows; a warp whose wait gave up scores its tile
-// +inf, marks the instance's status word and leaves the loop.
+// the candidates generated before the launch.
 //
 // The bodies are inlined into the kernel: as separate functions their
 // arguments went through a 240-byte stack frame and the launch was 7-8 %
@@ -35,6 +33,7 @@
 // SM ran different bodies at once, half of their stall samples were
 // instruction fetches, and the iteration took 3.5 ms; tiles are therefore
 // taken group by group (longest group first, longest tiles first within it).
+#include <algorithm>
 #include <map>
 #include <mutex>
 
@@ -45,25 +44,6 @@ namespace mtp {
 namespace {
 
 constexpr int kPersistThreads = 128;
-constexpr int kPersistChunk = 4;  // horizon chunk of a staged tile
-
-template <int NL, int T>
-__device__ __forceinline__ bool persist_chain(const RolloutArgs& a, const ChainModel& m, int r, bool live,
-                                           uint64_t* bars, float* buf, int& seq) {
-  if constexpr (T == 0) {
-    (void)bars;
-    (void)buf;
-    (void)seq;
-    if (!live) return true;
-    return rollout_chain_body<NL, kPrefetchBatch, 0>(a, m, r, true, nullptr);
-  } else {
-    StagedRows<NL, T> st;
-    st.attach(bars, buf, live ? a.U + (size_t)r * a.H * NL : nullptr, a.H, seq);
-    const bool ok = rollout_chain_body<NL, kPrefetchBatch, T>(a, m, r, live, &st);
-    seq = st.seq;
-    return __all_sync(0xffffffffu, ok);
-  }
-}
 
 template <int K>
 __device__ __forceinline__ void pm_item(int k, const RolloutArgs& a, const PointMassModel& m, int r0, float* buf) {
@@ -74,15 +54,18 @@ __device__ __forceinline__ void pm_item(int k, const RolloutArgs& a, const Point
 }
 
 template <int NL>
-__device__ __forceinline__ bool chain_tile(int links, bool staged, const RolloutArgs& a, const ChainModel& m,
-                                           int r, bool live, uint64_t* bars, float* buf, int& seq) {
+__device__ __forceinline__ void chain_item(int links, bool staged, const RolloutArgs& a, const ChainModel& m, int r0,
+                                           float* buf) {
   if constexpr (NL <= kPersistMaxLinks) {
-    if (links == NL)
-      return staged ? persist_chain<NL, kPersistChunk>(a, m, r, live, bars, buf, seq)
-                    : persist_chain<NL, 0>(a, m, r, live, bars, buf, seq);
-    return chain_tile<NL + 1>(links, staged, a, m, r, live, bars, buf, seq);
-  } else {
-    return false;
+    if (links != NL) return chain_item<NL + 1>(links, staged, a, m, r0, buf);
+    const int r = r0 + (threadIdx.x & 31);
+    if (staged) {
+      constexpr int T = chain_chunk(NL);
+      const StagedRows<NL, T> st{a.U + (size_t)r0 * a.H * NL, min(32, a.rows - r0), buf};
+      rollout_chain_body<NL, kPrefetchBatch, T>(a, m, r, r < a.rows, &st);
+    } else if (r < a.rows) {
+      rollout_chain_body<NL, kPrefetchBatch, 0>(a, m, r, true, nullptr);
+    }
   }
 }
 
@@ -90,11 +73,7 @@ __global__ void __launch_bounds__(kPersistThreads, 3) k_rollout_persistent(const
   __shared__ PointMassModel models[kPersistThreads / 32];
   extern __shared__ __align__(16) unsigned char persist_smem[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  unsigned char* area = persist_smem + (size_t)warp * p.warp_bytes;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(area);
-  float* buf = reinterpret_cast<float*>(area + 16);
-  init_stage_bars(bars);
-  int seq = 0;
+  float* const buf = reinterpret_cast<float*>(persist_smem + (size_t)warp * p.warp_bytes);
   for (;;) {
     int w = 0;
     if (lane == 0) w = (int)atomicAdd(p.head, 1u);
@@ -113,19 +92,15 @@ __global__ void __launch_bounds__(kPersistThreads, 3) k_rollout_persistent(const
     const RolloutArgs a = p.ra[__ldg(p.order + lo)];
     const int r0 = (w - __ldg(p.wstart + lo)) * 32;
     const int dim = (code >> 8) & 0xff;
-    bool ok = true;
     if ((code & 0xff) == MTP_DYN_POINTMASS) {
       load_pm_model(models[warp], p.pm[model]);
       pm_item<1>(dim, a, models[warp], r0, buf);
     } else {
-      const int r = r0 + lane;
       const ChainModel cm = p.cm[model];
       // staged only where the instance's rows allow it and the launch asks for it
-      ok = chain_tile<1>(dim, p.staged && (code >> 16) != 0, a, cm, r, r < a.rows, bars, buf, seq);
+      chain_item<1>(dim, p.staged && (code >> 16) != 0, a, cm, r0, buf);
     }
-    // the model slot and the staging buffers are reused by the next item
-    __syncwarp();
-    if (!__all_sync(0xffffffffu, ok)) break;
+    __syncwarp();  // the model slot and the staging buffers are reused by the next item
   }
 }
 
@@ -138,14 +113,14 @@ static size_t pm_floats_of(int k) {
 }
 size_t persist_pm_floats(int axes) { return pm_floats_of<1>(axes); }
 
+template <int NL>
+static size_t chain_bytes_of(int links) {
+  if constexpr (NL <= kPersistMaxLinks)
+    return std::max(NL <= links ? StageShape<NL, chain_chunk(NL)>::kWarpBytes : size_t(0), chain_bytes_of<NL + 1>(links));
+  else return 0;
+}
 size_t persist_warp_bytes(size_t pm_floats, int max_links_staged) {
-  size_t f = pm_floats;
-  if (max_links_staged > 0) {
-    const int quads = (kPersistChunk * max_links_staged + 3) / 4;
-    const int stride = 4 * (quads % 2 ? quads : quads + 1);
-    f = std::max(f, (size_t)2 * 32 * stride);
-  }
-  return 16 + f * sizeof(float);
+  return std::max({pm_floats * sizeof(float), chain_bytes_of<1>(max_links_staged), size_t(16)});
 }
 
 int persist_blocks_per_sm(size_t warp_bytes) {

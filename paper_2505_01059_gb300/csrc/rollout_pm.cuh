@@ -37,11 +37,6 @@ constexpr int kPmThreads = 128;  // at most four warps per block
 constexpr int kMaxPmAxes = 16;
 constexpr int kPmSmemMax = 68 * 1024;  // dynamic shared memory of a block, at most
 
-__device__ __forceinline__ void copy_async_16(float* smem_dst, const float* gmem_src) {
-  const unsigned dst = (unsigned)__cvta_generic_to_shared(smem_dst);
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(gmem_src) : "memory");
-}
-
 // Copies an instance's model to this warp's slot in shared memory.
 __device__ __forceinline__ void load_pm_model(PointMassModel& m, const PointMassModel& src) {
   const int* s = reinterpret_cast<const int*>(&src);
@@ -133,29 +128,31 @@ __device__ __forceinline__ void load_steps(const float* p, float (&u)[N]) {
   }
 }
 
-// Asynchronous copies, by one warp, of n candidates' next `steps` steps of
-// controls (src, H K floats apart) into rows `row` floats apart whose steps are
-// KS floats apart: in 16-byte pieces (vec: every piece aligned, and inside one
-// step where KS is not K) or by single floats.
+// copy_controls into rows whose steps are KS floats apart (a 16-byte piece lies
+// inside one step where KS is not K).
 template <int K, int KS>
-__device__ __forceinline__ void copy_controls(const float* src, int H, int n, int steps, bool vec, float* dst, int row) {
-  const int lane = threadIdx.x & 31;
-  const int len = vec ? steps * K / 4 : steps * K;  // pieces per candidate
-  int i = lane / len, o = lane - i * len;
-  const int di = 32 / len, dlen = 32 - di * len;
-  while (i < n) {
-    const int f = vec ? 4 * o : o;
-    const int at = KS == K ? f : f / K * KS + f % K;
-    if (vec) copy_async_16(dst + i * row + at, src + (size_t)i * H * K + f);
-    else copy_async_f32(dst + i * row + at, src + (size_t)i * H * K + f);
-    i += di;
-    o += dlen;
-    if (o >= len) {
-      o -= len;
-      ++i;
+__device__ __forceinline__ void copy_steps(const float* src, int H, int n, int steps, bool vec, float* dst, int row) {
+  if constexpr (KS == K) {
+    copy_controls<K>(src, H, n, steps, vec, dst, row);
+  } else {
+    const int lane = threadIdx.x & 31;
+    const int len = vec ? steps * K / 4 : steps * K;  // pieces per candidate
+    int i = lane / len, o = lane - i * len;
+    const int di = 32 / len, dlen = 32 - di * len;
+    while (i < n) {
+      const int f = vec ? 4 * o : o;
+      const int at = f / K * KS + f % K;
+      if (vec) copy_async_16(dst + i * row + at, src + (size_t)i * H * K + f);
+      else copy_async_f32(dst + i * row + at, src + (size_t)i * H * K + f);
+      i += di;
+      o += dlen;
+      if (o >= len) {
+        o -= len;
+        ++i;
+      }
     }
+    copy_async_commit();
   }
-  copy_async_commit();
 }
 
 // Whether an instance's control rows can be copied in 16-byte pieces.
@@ -193,7 +190,7 @@ __device__ __forceinline__ void rollout_pm_lanes(const RolloutArgs& a, const Poi
   const float dt = a.dt;
   const float w_ctrl = pm.w_ctrl;
   auto request = [&](int t0) {
-    if (t0 < H) copy_controls<K, K>(U + (size_t)t0 * K, H, n, min(T, H - t0), vec, sm + (t0 / T & 1) * T * K, row);
+    if (t0 < H) copy_controls<K>(U + (size_t)t0 * K, H, n, min(T, H - t0), vec, sm + (t0 / T & 1) * T * K, row);
   };
   float total = 0.f;
   for (int mdl = 0; mdl < models; ++mdl) {
@@ -257,7 +254,7 @@ __device__ __forceinline__ void rollout_pm_lanes(const RolloutArgs& a, const Poi
 
 // The lane body's steps in flight and chunk length: more steps where a position
 // takes few registers, and as long a chunk as kPmLaneFloats hold.
-constexpr int kPmLaneFloats = 4224;
+constexpr int kPmLaneFloats = 4352;
 template <int K>
 struct PmLane {
   static constexpr int P = K <= 4 ? 4 : 2;
@@ -340,7 +337,7 @@ __device__ __forceinline__ void rollout_pm_tile(const RolloutArgs& a, const Poin
   float* const cst = G + C * K;
   const int ld = T + 1;  // odd: pass 3's lanes read distinct banks
   auto request = [&](int t0, int buf) {
-    copy_controls<K, KS>(U + (size_t)t0 * K, H, n, min(T, H - t0), vec, sm + buf * C * row, row);
+    copy_steps<K, KS>(U + (size_t)t0 * K, H, n, min(T, H - t0), vec, sm + buf * C * row, row);
   };
   float total = 0.f;
   for (int mdl = 0; mdl < models; ++mdl) {

@@ -57,7 +57,6 @@ struct mtp_handle {
   float* x0 = nullptr;
   float* Z = nullptr;  // (M, N, n) graph of the current iteration (bfloat16 when tc_graph)
   uint32_t* status = nullptr;  // device status word: bits a rollout sets when a bounded wait gave up
-  int rollout_chunk = 0;       // horizon chunk of the staged control loads of a lone rollout (0: direct)
   bool tc_graph = false;       // graph rows contracted on the tensor cores (BF16 B-spline)
   double* entropy = nullptr;   // last iteration's cost entropy (MTP_FLAG_COST_ENTROPY)
   // two-stage elite selection (B beyond one block): chunk length, chunk

@@ -420,7 +420,7 @@ cudaError_t launch_rollout(const mtp_handle* h, const RolloutArgs& a, cudaStream
   const mtp_problem& p = h->pr;
   if (p.dyn == MTP_DYN_POINTMASS) return launch_rollout_pointmass(a, pointmass_model(p), s);
   if (p.dyn == MTP_DYN_LEGGED) return launch_rollout_legged(a, legged_model(p), p.n_links, s);
-  return launch_rollout_chain(a, chain_model(p), p.n_links, h->rollout_chunk, s);
+  return launch_rollout_chain(a, chain_model(p), p.n_links, s);
 }
 
 // Stage event: inside a stream capture it must be an external event record

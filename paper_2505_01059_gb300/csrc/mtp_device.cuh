@@ -204,12 +204,11 @@ constexpr uint32_t kStatusTcTimeout = 2u;
 // take 17 KB (what lets three persistent CTAs share an SM), else 4.
 __host__ __device__ constexpr int chain_chunk(int links) { return links <= 8 ? 8 : 4; }
 
-// Whether a rollout launch may stage its controls through shared memory with
-// 16-byte copies (see StagedRows): 16-byte aligned rows of a multiple of 4
-// floats, one model per candidate, no state output.
+// Whether a chain's rollout launch may stage its controls through shared memory
+// (see StagedRows): 16-byte aligned rows of a multiple of 4 floats, no state
+// output.
 inline bool can_stage(const RolloutArgs& a, int k) {
-  return a.X == nullptr && a.dr_mode != MTP_DR_SHARED &&
-         ((uintptr_t)a.U % 16u) == 0 && ((long long)a.H * k) % 4 == 0;
+  return a.X == nullptr && ((uintptr_t)a.U % 16u) == 0 && ((long long)a.H * k) % 4 == 0;
 }
 
 // The obstacle centres first and the struct 16-byte aligned: each centre
@@ -282,15 +281,15 @@ cudaError_t launch_candidates(const CandArgs& a, int local_blocks, cudaStream_t 
 cudaError_t launch_sample_tensor(const Dims& dm, Key key, uint32_t iter, const float* umin,
                                  const float* umax, float* Z, int32_t* I, float* C,
                                  cudaStream_t s);
-// Rollouts: with `chunk` a chain's controls are staged chain_chunk steps at a
-// time (0, or a launch that cannot stage, loads directly).
+// Rollouts: a chain's controls are staged chain_chunk steps at a time or loaded
+// directly, as launch_rollout_chain's rule or a batch group's `chunk` (0:
+// directly) says; a launch that cannot stage loads directly.
 cudaError_t init_rollout_pm_attributes();
 cudaError_t init_rollout_chain_attributes();
 cudaError_t init_rollout_pm_batch_attributes();
 cudaError_t init_rollout_chain_batch_attributes();
 cudaError_t launch_rollout_pointmass(const RolloutArgs& a, const PointMassModel& m, cudaStream_t s);
-cudaError_t launch_rollout_chain(const RolloutArgs& a, const ChainModel& m, int links, int chunk,
-                                 cudaStream_t s);
+cudaError_t launch_rollout_chain(const RolloutArgs& a, const ChainModel& m, int links, cudaStream_t s);
 cudaError_t launch_rollout_legged(const RolloutArgs& a, const LeggedModel& m, int links,
                                   cudaStream_t s);
 cudaError_t launch_rollout_legged_batch(const RolloutArgs* d_ra, const LeggedModel* d_lm,

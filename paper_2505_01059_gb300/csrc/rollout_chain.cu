@@ -15,11 +15,11 @@ cudaError_t chain_launch(const RolloutArgs& a, const ChainModel& m, cudaStream_t
 }
 
 template <int NL>
-cudaError_t chain_dispatch(const RolloutArgs& a, const ChainModel& m, int links, int chunk,
+cudaError_t chain_dispatch(const RolloutArgs& a, const ChainModel& m, int links, bool staged,
                            cudaStream_t s) {
   if constexpr (NL <= kMaxChainLinks) {
-    if (links == NL) return chunk ? chain_launch<NL, chain_chunk(NL)>(a, m, s) : chain_launch<NL, 0>(a, m, s);
-    return chain_dispatch<NL + 1>(a, m, links, chunk, s);
+    if (links == NL) return staged ? chain_launch<NL, chain_chunk(NL)>(a, m, s) : chain_launch<NL, 0>(a, m, s);
+    return chain_dispatch<NL + 1>(a, m, links, staged, s);
   } else {
     return cudaErrorInvalidValue;
   }
@@ -41,11 +41,20 @@ cudaError_t chain_attributes() {
 
 cudaError_t init_rollout_chain_attributes() { return chain_attributes<1>(); }
 
-cudaError_t launch_rollout_chain(const RolloutArgs& a, const ChainModel& m, int links, int chunk,
-                                 cudaStream_t s) {
+// Direct loads two steps ahead, or staged ones?  A lone warp per SM sub-partition
+// waits for its longest chain of instructions either way, and which form's code
+// is the shorter one was measured (us, direct / staged, 128 steps of 4096
+// candidates or 64 of 2048): 3 links 32.0 / 25.7, 4 links 30.6 / 35.2, 5 links
+// 27 / 34 (2048, 100 steps), 7 links 50 / 58, 9 links 85 / 90, 10 links 53 / 47, 12
+// links 54 / 53.  Once several warps share a sub-partition, staged: its loads are
+// coalesced (16384 candidates, 7 links: 65 / 59).
+static bool stages_alone(int links, int rows) {
+  return links <= 3 || links >= 10 || rows > 96 * device_sms();
+}
+
+cudaError_t launch_rollout_chain(const RolloutArgs& a, const ChainModel& m, int links, cudaStream_t s) {
   if (a.rows <= 0) return cudaSuccess;
-  if (!can_stage(a, links)) chunk = 0;
-  return chain_dispatch<1>(a, m, links, chunk, s);
+  return chain_dispatch<1>(a, m, links, can_stage(a, links) && stages_alone(links, a.rows), s);
 }
 
 int rollout_blocks(int rows) {

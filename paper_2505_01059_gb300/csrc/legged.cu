@@ -13,9 +13,9 @@
 // register Cholesky applies; p'' = (R_p - sum_j lb_j e'_j phi''_j) / m.
 // Contact forces at the 17 link end points enter through suffix sums (a
 // force at the distal end of link c acts on every phi_j with j <= c), the
-// velocity terms through the O(L) prefix / suffix form.  Per-thread vectors
-// (angles, velocities, sines, cosines, per-sample constants) are staged in
-// shared memory so the 16 x 16 factor fits the register file.
+// velocity terms through the O(L) prefix / suffix form.  What a thread keeps
+// from step to step (angles, velocities, per-sample constants) lies in shared
+// memory; a step's own vectors in registers.
 #include "rollout_common.cuh"
 
 namespace mtp {
@@ -45,9 +45,7 @@ __device__ __forceinline__ void rollout_legged_body(const RolloutArgs& a, const 
   float* LB = my + 4 * NL * BD;
   float* WV = my + 5 * NL * BD;
   float* SD = my + 6 * NL * BD;
-  float* SA = my + 7 * NL * BD;  // velocity-term suffix sums
-  float* SB = my + 8 * NL * BD;
-  float* TN = my + 9 * NL * BD;  // torques of steps t and t + 1 (two slots of NC)
+  float* TN = my + 7 * NL * BD;  // torques of steps t and t + 1 (two slots of NC)
 
   const int b = a.row0 + r;
   const uint32_t iter = a.d_iter ? *a.d_iter : a.iter;
@@ -113,12 +111,17 @@ __device__ __forceinline__ void rollout_legged_body(const RolloutArgs& a, const 
       float tau[NC];
 #pragma unroll
       for (int j = 0; j < NC; ++j) tau[j] = slot[j * BD];
+      // up to the factorisation a step's vectors stay in registers (the factor's
+      // own take their place); shared memory keeps the sines and cosines for the
+      // base acceleration after it
+      float c[NL], s[NL], om[NL], lb[NL];
 #pragma unroll
       for (int j = 0; j < NL; ++j) {
-        float sj, cj;
-        sincos_reduced(PHI[j * BD], &sj, &cj);
-        SN[j * BD] = sj;
-        CS[j * BD] = cj;
+        sincos_reduced(PHI[j * BD], &s[j], &c[j]);
+        SN[j * BD] = s[j];
+        CS[j * BD] = c[j];
+        om[j] = OMG[j * BD];
+        lb[j] = LB[j * BD];
       }
       // stage cost c(x_t, u_t): height, pitch and forward velocity of the
       // base link plus the torque penalty
@@ -136,32 +139,32 @@ __device__ __forceinline__ void rollout_legged_body(const RolloutArgs& a, const 
       for (int j = 0; j < NL; ++j) {
         const float tj = (j >= 1) ? tau[j - 1] : 0.f;
         const float tj1 = (j + 1 <= NC) ? tau[j] : 0.f;
-        rhs[j] = fmaf(-lm.gravity * LB[j * BD], CS[j * BD], tj - tj1);
+        rhs[j] = fmaf(-lm.gravity * lb[j], c[j], tj - tj1);
       }
       // contact: walk from the tip back to the base, accumulating the force
       // sum over the points beyond each link
       float cx = px, cy = py, cvx = vx, cvy = vy;
 #pragma unroll
       for (int j = 0; j < NL; ++j) {
-        const float l = lm.length[j], w = OMG[j * BD];
-        cx = fmaf(l, CS[j * BD], cx);
-        cy = fmaf(l, SN[j * BD], cy);
-        cvx = fmaf(-l * w, SN[j * BD], cvx);
-        cvy = fmaf(l * w, CS[j * BD], cvy);
+        const float l = lm.length[j], w = om[j];
+        cx = fmaf(l, c[j], cx);
+        cy = fmaf(l, s[j], cy);
+        cvx = fmaf(-l * w, s[j], cvx);
+        cvy = fmaf(l * w, c[j], cvy);
       }
       float Fx = 0.f, Fy = 0.f;
 #pragma unroll
-      for (int c = NL; c >= 0; --c) {
+      for (int point = NL; point >= 0; --point) {
         // branch-free: a point above the ground gets a zero normal force (a
         // divergent branch per point cost more than the arithmetic it skipped)
         const float fn_in = fmaxf(fmaf(-lm.k_contact, cy, -lm.c_contact * cvy), 0.f);
         const float fn = cy < 0.f ? fn_in : 0.f;
         Fx = fmaf(-mu_s * fn, smooth_sign(cvx * lm.inv_v_slip), Fx);
         Fy += fn;
-        if (c >= 1) {
-          const int j = c - 1;
-          const float l = lm.length[j], w = OMG[j * BD];
-          const float sj = SN[j * BD], cj = CS[j * BD];
+        if (point >= 1) {
+          const int j = point - 1;
+          const float l = lm.length[j], w = om[j];
+          const float sj = s[j], cj = c[j];
           rhs[j] = fmaf(l, fmaf(-sj, Fx, cj * Fy), rhs[j]);
           cx = fmaf(-l, cj, cx);
           cy = fmaf(-l, sj, cy);
@@ -173,34 +176,34 @@ __device__ __forceinline__ void rollout_legged_body(const RolloutArgs& a, const 
       // sums), and the base equation's right-hand side
       float Rx = Fx, Ry = fmaf(-m_tot, lm.gravity, Fy);
       {
-        float Sa = 0.f, Sb = 0.f;
+        float Sa[NL], Sb[NL];  // sums over the links beyond
+        float sum_a = 0.f, sum_b = 0.f;
 #pragma unroll
         for (int k = NL - 1; k >= 0; --k) {
-          SA[k * BD] = Sa;
-          SB[k * BD] = Sb;
-          const float w2 = OMG[k * BD] * OMG[k * BD];
-          Sa = fmaf(LB[k * BD], CS[k * BD] * w2, Sa);
-          Sb = fmaf(LB[k * BD], SN[k * BD] * w2, Sb);
+          Sa[k] = sum_a;
+          Sb[k] = sum_b;
+          const float w2 = om[k] * om[k];
+          sum_a = fmaf(lb[k], c[k] * w2, sum_a);
+          sum_b = fmaf(lb[k], s[k] * w2, sum_b);
         }
-        Rx += Sa;  // sum_j lb_j cos(phi_j) w_j^2
-        Ry += Sb;  // sum_j lb_j sin(phi_j) w_j^2
+        Rx += sum_a;  // sum_j lb_j cos(phi_j) w_j^2
+        Ry += sum_b;  // sum_j lb_j sin(phi_j) w_j^2
         float Pa = 0.f, Pb = 0.f;
 #pragma unroll
         for (int j = 0; j < NL; ++j) {
-          const float l = lm.length[j], lb = LB[j * BD];
-          const float sj = SN[j * BD], cj = CS[j * BD];
-          const float ca = fmaf(lb, Pa, l * SA[j * BD]);
-          const float cb = fmaf(lb, Pb, l * SB[j * BD]);
-          rhs[j] = rhs[j] - fmaf(sj, ca, -cj * cb);
-          const float w2 = OMG[j * BD] * OMG[j * BD];
-          Pa = fmaf(l, cj * w2, Pa);
-          Pb = fmaf(l, sj * w2, Pb);
+          const float l = lm.length[j];
+          const float ca = fmaf(lb[j], Pa, l * Sa[j]);
+          const float cb = fmaf(lb[j], Pb, l * Sb[j]);
+          rhs[j] = rhs[j] - fmaf(s[j], ca, -c[j] * cb);
+          const float w2 = om[j] * om[j];
+          Pa = fmaf(l, c[j] * w2, Pa);
+          Pb = fmaf(l, s[j] * w2, Pb);
         }
       }
       // Schur right-hand side
 #pragma unroll
       for (int j = 0; j < NL; ++j)
-        rhs[j] = fmaf(-LB[j * BD] * invm, fmaf(-SN[j * BD], Rx, CS[j * BD] * Ry), rhs[j]);
+        rhs[j] = fmaf(-lb[j] * invm, fmaf(-s[j], Rx, c[j] * Ry), rhs[j]);
       // Schur system S phi'' = rhs.  Below the diagonal S_jk = u_j . v_k with
       // u_j = lb_j (cos phi_j, sin phi_j) and v_k = WV_k (cos phi_k, sin phi_k):
       // a rank-2 semiseparable matrix plus its diagonal SD.  Its Cholesky
@@ -214,9 +217,9 @@ __device__ __forceinline__ void rollout_legged_body(const RolloutArgs& a, const 
         float m11 = 0.f, m12 = 0.f, m22 = 0.f;
 #pragma unroll
         for (int k = 0; k < NL; ++k) {
-          const float ck = CS[k * BD], sk = SN[k * BD], lbk = LB[k * BD], wvk = WV[k * BD];
-          u1[k] = lbk * ck;
-          u2[k] = lbk * sk;
+          const float ck = c[k], sk = s[k], wvk = WV[k * BD];
+          u1[k] = lb[k] * ck;
+          u2[k] = lb[k] * sk;
           const float mu1 = fmaf(m11, u1[k], m12 * u2[k]);
           const float mu2 = fmaf(m12, u1[k], m22 * u2[k]);
           const float inv = rsqrtf(SD[k * BD] - fmaf(u1[k], mu1, u2[k] * mu2));
@@ -290,7 +293,7 @@ __device__ __forceinline__ void rollout_legged_body(const RolloutArgs& a, const 
 template <int NL>
 __global__ void __launch_bounds__(kLegThreads) k_rollout_legged(const RolloutArgs a,
                                                                 const LeggedModel lm) {
-  __shared__ float sh[(9 * NL + 2 * (NL - 1)) * kLegThreads];
+  __shared__ float sh[(7 * NL + 2 * (NL - 1)) * kLegThreads];
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= a.rows) return;
   rollout_legged_body<NL>(a, lm, r, sh + threadIdx.x);
@@ -300,7 +303,7 @@ template <int NL>
 __global__ void __launch_bounds__(kLegThreads) k_rollout_legged_batch(
     const RolloutArgs* __restrict__ ra, const LeggedModel* __restrict__ lms,
     const int* __restrict__ row_start, int count) {
-  __shared__ float sh[(9 * NL + 2 * (NL - 1)) * kLegThreads];
+  __shared__ float sh[(7 * NL + 2 * (NL - 1)) * kLegThreads];
   const int g = blockIdx.x * blockDim.x + threadIdx.x;
   if (g >= __ldg(row_start + count)) return;
   const int i = batch_instance(row_start, count, g);

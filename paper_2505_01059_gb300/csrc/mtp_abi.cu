@@ -379,20 +379,26 @@ cudaError_t launch_generate(const mtp_handle* h, CandArgs& c, cudaStream_t s) {
   const bool tc = c.graph_blocks > 0 && h->tc_graph && bspline_tc_eligible(c);
   const int local_blocks = c.U_local ? local_blocks_for(h, (long long)c.local_rows + 1) : 0;
   if (tc && h->side && !h->pipeline && local_blocks > 0) {
-    // the graph (its Z, then the tensor-core rows) on the side stream beside
-    // the local rows and the mean row: they write disjoint rows of U.  On the
-    // 16-link legged workload this took generation from 183 to about 120 us
-    // (the serial launches left the tensor-core rows on the critical path)
+    // the tensor-core rows beside the local rows and the mean row on the side
+    // stream: they write disjoint rows of U.  The local rows wait for the graph
+    // too, so that the contraction, launched first, finds room (started at once
+    // they fill every SM and it runs after them).  One after the other -> beside
+    // each other, 16384 candidates of 256 x 15 with beta 0.2 / 0.3 / 0.6: 85 / 83 /
+    // 72 -> 82 / 79 / 67 us replayed and 92 / 90 / 78 -> 88 / 85 / 74 called one by
+    // one, 1000 of 100 x 5: 10.5 -> 7.6 and 16.4 -> 13.8.  Two or three of the
+    // contraction's CTAs per SM instead of four replay up to 3 % faster but take
+    // up to 17 % longer in single calls, where the local rows start later.
     cudaError_t e;
-    if ((e = cudaEventRecord(h->ev_fork, s)) || (e = cudaStreamWaitEvent(h->side, h->ev_fork, 0))) return e;
     if (!c.C_in) {
       c.Z_global = h->Z;
-      if ((e = launch_graph_Z(c, h->Z, h->side))) return e;
+      if ((e = launch_graph_Z(c, h->Z, s))) return e;
     }
-    if ((e = launch_bspline_tc(c, h->side)) || (e = cudaEventRecord(h->ev_join, h->side))) return e;
+    if ((e = cudaEventRecord(h->ev_fork, s)) || (e = cudaStreamWaitEvent(h->side, h->ev_fork, 0)) ||
+        (e = launch_bspline_tc(c, s)))
+      return e;
     CandArgs local = c;
     local.graph_blocks = 0;
-    if ((e = launch_candidates(local, local_blocks, s))) return e;
+    if ((e = launch_candidates(local, local_blocks, h->side)) || (e = cudaEventRecord(h->ev_join, h->side))) return e;
     return cudaStreamWaitEvent(s, h->ev_join, 0);
   }
   if (c.graph_blocks > 0 && (h->global_Z || tc) && !c.C_in) {
@@ -837,6 +843,8 @@ mtp_status mtp_sample_local(mtp_handle* h, uint32_t iter, float* d_U, void* stre
   return MTP_OK;
 }
 
+static void ensure_side(mtp_handle* h);
+
 mtp_status mtp_generate_candidates(mtp_handle* h, uint32_t iter, float* d_U, void* stream) {
   if (!h || !d_U) return fail(h, MTP_ERR_INVALID_ARG, "generate_candidates: bad argument");
   DeviceGuard g(h->device);
@@ -849,6 +857,7 @@ mtp_status mtp_generate_candidates(mtp_handle* h, uint32_t iter, float* d_U, voi
   c.U_local = d_U;
   c.local_rows = dm.L;
   c.U_mean = d_U + Hn * (dm.B - 1);
+  ensure_side(h);
   cudaError_t e = launch_generate(h, c, (cudaStream_t)stream);
   if (e != cudaSuccess) return cuda_fail(h, e, "generate_candidates");
   return MTP_OK;
@@ -925,26 +934,33 @@ static mtp_status read_stage_events(mtp_handle* h, const cudaEvent_t* ev, double
   return MTP_OK;
 }
 
+// A tensor-core handle's side stream (launch_generate), made by the first call
+// that uses it; without it the rows are made one after the other, with the same
+// bits.
+static void ensure_side(mtp_handle* h) {
+  if (!h->tc_graph || h->pipeline || h->side) return;
+  // a capture elsewhere in the process is not disturbed by it
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  if (cudaStreamCreateWithFlags(&h->side, cudaStreamNonBlocking) != cudaSuccess ||
+      cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
+      cudaEventCreateWithFlags(&h->ev_join, cudaEventDisableTiming) != cudaSuccess) {
+    cudaGetLastError();
+    if (h->side) cudaStreamDestroy(h->side);
+    if (h->ev_fork) cudaEventDestroy(h->ev_fork);
+    if (h->ev_join) cudaEventDestroy(h->ev_join);
+    h->side = nullptr;
+    h->ev_fork = h->ev_join = nullptr;
+  }
+  cudaThreadExchangeStreamCaptureMode(&mode);
+}
+
 // The pipeline's second candidate buffer, stream and events, made by the
 // first single-instance plan step that uses them (a handle planned only in
 // batches never needs them).  If they cannot be made the handle plans
 // without the pipeline, which gives the same results.
 static void ensure_pipeline(mtp_handle* h) {
-  if (h->tc_graph && !h->pipeline && !h->side) {
-    // a tensor-core handle's side stream for its graph rows (launch_generate);
-    // without it the rows are made after the local rows, with the same bits
-    if (cudaStreamCreateWithFlags(&h->side, cudaStreamNonBlocking) != cudaSuccess ||
-        cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&h->ev_join, cudaEventDisableTiming) != cudaSuccess) {
-      cudaGetLastError();
-      if (h->side) cudaStreamDestroy(h->side);
-      if (h->ev_fork) cudaEventDestroy(h->ev_fork);
-      if (h->ev_join) cudaEventDestroy(h->ev_join);
-      h->side = nullptr;
-      h->ev_fork = h->ev_join = nullptr;
-    }
-    return;
-  }
+  ensure_side(h);
   if (!h->pipeline || h->side) return;
   const size_t n = (size_t)h->dm.H * h->dm.n * h->dm.B;
   if (dalloc(&h->Ubuf[1], n) != cudaSuccess ||

@@ -133,7 +133,8 @@ typedef struct mtp_sizes {
                                     the first, when pipelined) */
   int32_t pipelined;             /* mtp_plan_step prepares each next iteration's graph rows
                                     (1) or graph rows and local draws (2) on the SMs its
-                                    rollout leaves idle; 0: not pipelined */
+                                    rollout (a point mass: its selection) leaves idle; 0:
+                                    not pipelined */
 } mtp_sizes;
 
 /* Device buffers owned by a handle (valid until mtp_destroy).  After
@@ -229,7 +230,8 @@ mtp_status mtp_elite_update(mtp_handle* h, const float* d_cost, const float* d_U
  * MTP_FLAG_NO_GRAPH is set.  On a pipelined handle (mtp_sizes.pipelined)
  * each iteration also prepares the next iteration's graph rows (and, with
  * enough idle SMs, its local draws) on a second stream, on the SMs the
- * rollout leaves idle, and the next iteration (in this call or the next,
+ * rollout leaves idle (a point mass: after its rollout, beside the
+ * selection's one block), and the next iteration (in this call or the next,
  * unless mtp_set_state or a batch run changed the iteration counter in
  * between) only makes or finishes its local rows and mean row.  The results
  * are the same bits as without the pipeline. */
@@ -254,12 +256,12 @@ mtp_status mtp_shift(mtp_handle* h, int32_t k, void* stream);
  * Synchronises the device. */
 mtp_status mtp_cost_entropy(mtp_handle* h, double* h_entropy);
 
-/* Device-side failures since the last call: the rollouts stage their controls
- * through shared memory with bulk copies and wait for them with a bounded
- * wait (about two seconds); a wait that gives up marks the handle and scores
- * its candidates +inf instead of hanging the GPU.  Synchronises the device,
- * then returns MTP_ERR_TIMEOUT (and clears the mark) if that happened in any
- * of the handle's rollouts (alone or in a batch), else MTP_OK. */
+/* Device-side failures since the last call: the tensor-core contraction of the
+ * graph rows waits for its MMAs with a bounded wait (about two seconds); a
+ * wait that gives up marks the handle and leaves those rows unwritten instead
+ * of hanging the GPU.  Synchronises the device, then returns MTP_ERR_TIMEOUT
+ * (and clears the mark) if that happened in any of the handle's generations
+ * (alone or in a batch), else MTP_OK. */
 mtp_status mtp_device_status(mtp_handle* h);
 
 /* Self-test of the bounded device waits: one warp waits on an mbarrier whose
@@ -336,9 +338,9 @@ mtp_status mtp_batch_plan_step(mtp_batch* b, const float* d_x0, int32_t iters, f
 /* Picks the rollout tile of each (dynamics, dimension) group by timing its
  * rollout launch (best of three) for every choice: threads per block (32, 64
  * or 128) and, for chains, the horizon chunk of the staged control loads (0:
- * direct loads; 4 steps of every candidate's controls copied at once into
- * shared memory by bulk copies, when every member's rows allow it: 16-byte
- * aligned, H * n a multiple of 4, one model per candidate).  The legged group
+ * direct loads; 8 steps of every candidate's controls, 4 from 9 links on,
+ * copied ahead into shared memory by asynchronous copies, when every member's
+ * rows allow it: 16-byte aligned, H * n a multiple of 4).  The legged group
  * keeps its fixed tile.  Writes (dynamics, dimension, block, chunk, candidates
  * per thread: 1) to tiles_out (5 * groups entries, may be NULL) and the number
  * of groups to n_groups.  Then it picks the rollout
@@ -362,9 +364,10 @@ mtp_status mtp_batch_autotune(mtp_batch* b, int32_t* tiles_out, int32_t* n_group
  *   warp takes warp tiles of 32 candidates of one instance from a device
  *   counter, group by group (the longest group first, within a group the
  *   longest expected rollout first: H times the group's time per step).
- *   A chain's controls are staged through shared memory 4 steps at a time
- *   where the instance's rows allow it (_STAGED) or loaded directly (_DIRECT).  Legged robots and longer chains keep their own launches
- *   beside it.  The launch is counted as one kernel by mtp_batch_launches.
+ *   A chain's controls are staged through shared memory (8 steps at a time, 4
+ *   for 9 links) where the instance's rows allow it (_STAGED) or loaded
+ *   directly (_DIRECT).  Legged robots and longer chains keep their own
+ *   launches beside it.  The launch is counted as one kernel by mtp_batch_launches.
  * MTP_BATCH_ROLLOUT_PERSISTENT_SPLIT: the same with staged tiles, in two
  *   persistent launches split at a group boundary near 65 % of the expected
  *   rollout work: the first starts as soon as its groups' candidates are made

@@ -528,8 +528,8 @@ __device__ __forceinline__ double canonical_sum(double (&part)[32 / G]) {
 }
 
 // Rounds of 32 elites whose loads the update issues together (measured on
-// the C1 point mass, E 32: 1 or 2 rounds 46.1 us per plan step, 4 rounds
-// 47.7; the 7-link arm, E 64, the same within 1 us for 1, 2 and 4).
+// the C1 point mass, E 32, when its plan step took 46 us: 1 or 2 rounds 46.1,
+// 4 rounds 47.7; the 7-link arm, E 64, the same within 1 us for 1, 2 and 4).
 constexpr int kUpdRounds = 2;
 
 // Threads per block of the update launches.
@@ -813,7 +813,7 @@ cudaError_t launch_select_batch(const SelectArgs* d_args, int count, size_t smem
 // instructions, a warp of 32 lane-wide elements therefore 30,000 cycles; 4 lanes
 // per element cut that to a quarter for about 4 % more instructions in all
 // (serving cycle of 48 robots: 48 -> 14 us per group of chains, the cycle 385 ->
-// 345 us).  More lanes while the launch leaves sub-partitions idle.
+// 345 us, since 314 by the chains' staging).  More lanes while the launch leaves sub-partitions idle.
 int update_lanes(long long elements) {
   int G = 4;
   const long long want = (long long)device_sms() * 256;

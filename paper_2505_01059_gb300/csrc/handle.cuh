@@ -38,14 +38,15 @@ struct mtp_handle {
   // makes the next iteration's graph rows (and, with many idle SMs, its
   // draws) on those SMs while its rollout runs (on `side`), into the other
   // candidate buffer; the next iteration then only makes (or finishes) its
-  // local rows and mean row.
+  // local rows and mean row.  A point mass's rollout is over in a few
+  // microseconds: it prepares after it, beside the selection's one block.
   bool pipeline = false;
   bool prep_local = false;    // the local draws are prepared too (else only the graph rows)
   float* Ubuf[2] = {nullptr, nullptr};
   int cur = 0;                // Ubuf[cur] holds the latest iteration's candidates
   bool prep_valid = false;    // Ubuf[cur ^ 1] holds the draws and graph rows of prep_iter
   uint32_t prep_iter = 0;
-  int prep_grid = 0;          // SMs the rollout leaves free
+  int prep_grid = 0;          // blocks of k_prepare: one per SM it may take
   int prep_spb = 1;           // graph paths per pass of a k_prepare block
   size_t prep_smem = 0;       // dynamic shared memory of a k_prepare block (a whole SM)
   cudaStream_t side = nullptr;
@@ -56,7 +57,7 @@ struct mtp_handle {
   float* ustar = nullptr;
   float* x0 = nullptr;
   float* Z = nullptr;  // (M, N, n) graph of the current iteration (bfloat16 when tc_graph)
-  uint32_t* status = nullptr;  // device status word: bits a rollout sets when a bounded wait gave up
+  uint32_t* status = nullptr;  // device status word: kStatusTcTimeout when a bounded wait gave up
   bool tc_graph = false;       // graph rows contracted on the tensor cores (BF16 B-spline)
   double* entropy = nullptr;   // last iteration's cost entropy (MTP_FLAG_COST_ENTROPY)
   // two-stage elite selection (B beyond one block): chunk length, chunk

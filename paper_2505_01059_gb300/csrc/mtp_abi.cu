@@ -588,7 +588,8 @@ int paths_per_block_for(const Dims& dm, int32_t interp, bool global_Z) {
 //    1.5-13 us per step (their finishing pass reads them back from DRAM,
 //    and 24 SMs prepare both in 80 us, longer than the rollout);
 //  - 2-D point mass, B 512 (136 idle SMs): preparing the draws too gains
-//    4-7 us per step.
+//    4-7 us per step (measured beside a 21 us rollout; the rule still counts
+//    the SMs that one block per 32 candidates would leave idle).
 constexpr int kMinPrepareSMs = 16;
 constexpr int kFullPrepareSMs = 64;
 

@@ -1,5 +1,5 @@
-// selftest.cu -- a self-test of the bounded device waits the rollouts and
-// the tensor-core contraction use: one warp waits on an mbarrier whose
+// selftest.cu -- a self-test of the bounded device wait that the
+// tensor-core contraction uses: one warp waits on an mbarrier whose
 // expected bytes never arrive (nothing copies into it), so the wait can only
 // end by giving up at its time limit; the kernel then reports that and
 // returns, and the context stays usable.

@@ -449,7 +449,7 @@ def mtp_selftest_bounded_wait(limit_s: float):
 
 def mtp_device_status(h: Handle):
     """Raises MtpError (MTP_ERR_TIMEOUT) if a bounded device wait of the
-    handle's rollouts gave up since the last check; synchronises."""
+    handle's tensor-core contraction gave up since the last check; synchronises."""
     _check(load_library().mtp_device_status(h.ptr), h.ptr)
 
 

@@ -613,6 +613,18 @@ bool tc_graph_rule(const mtp_problem& p, const Dims& dm) {
   return bspline_tc_eligible(probe);
 }
 
+// Whether a point mass's preparation is worth its place beside the selection: it
+// has to be over in the selection's 10 us, in one block per SM.  Microseconds per
+// iteration of ten, pipelined / not: Akima rows of 2 axes (B 2048, H 64) 22.4 /
+// 23.4, 4 (2048, 128) 27.2 / 27.1, 6 (2048, 128) 32.9 / 30.9, 12 (512, 128) 37.2 /
+// 30.1, 12 (1024, 200) 50.5 / 38.2; B-spline rows of 2 axes (512, 64) 21.0 / 23.3,
+// 4 (2048, 128) 32.2 / 34.3, 10 (2048, 100) 39.8 / 40.1, 8 (2500, 128) 44.6 / 44.3,
+// 12 (2048, 200) 60.8 / 59.4.
+bool prepares_beside_selection(const mtp_problem& p) {
+  if (p.interp == MTP_INTERP_AKIMA) return p.ctrl_dim < 4;
+  return (long long)p.B * p.horizon * p.ctrl_dim <= (1LL << 21);
+}
+
 cudaError_t pipeline_plan(const mtp_problem& p, const Dims& dm, int paths_per_block, bool* on,
                           bool* local, int* grid, size_t* smem, int* prep_spb) {
   *on = false;
@@ -632,6 +644,7 @@ cudaError_t pipeline_plan(const mtp_problem& p, const Dims& dm, int paths_per_bl
     return cudaSuccess;
   const int free_sms = sms - rollout_blocks(dm.B);
   if (free_sms < kMinPrepareSMs) return cudaSuccess;
+  if (p.dyn == MTP_DYN_POINTMASS && !prepares_beside_selection(p)) return cudaSuccess;
   const bool draws = free_sms >= kFullPrepareSMs && dm.L > 0;
   if (!draws && dm.P <= 0) return cudaSuccess;  // nothing to prepare
   CandArgs probe{};

@@ -55,11 +55,13 @@ __device__ __forceinline__ void dr_scales(const RolloutArgs& a, uint32_t iter, u
   }
 }
 
-// The nearest whole number (ties to even), by adding and taking off 1.5 * 2^23:
-// rintf's value below 2^22, without its place in the SFU's queue (8 cycles per
-// warp and operation, in front of the sines and cosines).
+// rintf for every x, by adding and taking off 2^23 (from there on x is whole):
+// without rintf's place in the SFU's queue (8 cycles per warp and operation, in
+// front of the sines and cosines).
 __device__ __forceinline__ float round_nearest(float x) {
-  return __fadd_rn(__fadd_rn(x, 12582912.f), -12582912.f);
+  const float a = fabsf(x);
+  const float r = copysignf(__fadd_rn(__fadd_rn(a, 8388608.f), -8388608.f), x);
+  return a < 8388608.f ? r : x;
 }
 
 // sin and cos of an absolute link angle: Cody-Waite reduction of x by 2 pi

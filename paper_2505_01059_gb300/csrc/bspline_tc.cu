@@ -19,8 +19,7 @@
 // steps, K = 16 per instruction) into tensor memory.  The B operand comes from
 // the handle's table in its shared-memory layout.  The products of two bfloat16 values are exact in FP32; the
 // sums are FP32.  In the epilogue warps w and w + 4 take the two halves of
-// quarter w's steps, 16 at a time with tcgen05.ld (the next 16 requested before
-// the current ones are used), clamp them to the control box and write them
+// quarter w's steps, 16 at a time with tcgen05.ld, clamp them to the control box and write them
 // through a per-warp shared-memory transpose: for each path, 16 steps x n
 // controls are one contiguous block of U, stored with 16-byte vector stores
 // whose places in the transpose and in U a lane computes once per instance.
@@ -177,12 +176,18 @@ __device__ __forceinline__ TcPlan tc_plan(TcSmem& S, const CandArgs& a) {
   return pl;
 }
 
+// Sixteen accumulator columns of this lane's row.  The load and the wait for it
+// are one statement: a register of the load means nothing before the wait, and
+// what names the registers in between (a merge with another path's, a hoisted
+// use) is the compiler's choice.
 __device__ __forceinline__ void tmem_load16(uint32_t taddr, uint32_t (&v)[16]) {
   asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
+      "tcgen05.wait::ld.sync.aligned;\n"
       : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
         "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-      : "r"(taddr));
+      : "r"(taddr)
+      : "memory");
 }
 
 // Path group g of one instance's graph rows, horizon slice s (the B operand
@@ -276,10 +281,9 @@ __device__ __forceinline__ bool tc_tile(TcSmem& S, const CandArgs& a, const TcPl
   float* mine = st + p * 16 * n + i;
   float* out = a.U_graph + (size_t)wb0 * Hn + (size_t)t_first * n;
   const uint32_t taddr = S.tmem_base + ((uint32_t)(32 * w) << 16) + (uint32_t)(64 * (warp >> 2));
-  uint32_t v[16];
-  if (t_first < t_end) tmem_load16(taddr, v);
   for (int t0 = t_first; t0 < t_end; t0 += 16, out += 16 * n) {
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+    uint32_t v[16];
+    tmem_load16(taddr + (uint32_t)(t0 - t_first), v);
     const int steps = min(16, H - t0);  // steps of this chunk inside the horizon
     __syncwarp();                        // the previous chunk's reads of st are done
     if (p < wpaths) {
@@ -287,7 +291,6 @@ __device__ __forceinline__ bool tc_tile(TcSmem& S, const CandArgs& a, const TcPl
       for (int tt = 0; tt < 16; ++tt) mine[tt * n] = clamp_box(__uint_as_float(v[tt]), lo, hi);
     }
     __syncwarp();
-    if (t0 + 16 < t_end) tmem_load16(taddr + (uint32_t)(t0 + 16 - t_first), v);
     if (vec && steps == 16) {
 #pragma unroll
       for (int z = 0; z < 4; ++z)
@@ -305,7 +308,6 @@ __device__ __forceinline__ bool tc_tile(TcSmem& S, const CandArgs& a, const TcPl
       }
     }
   }
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
   __syncwarp();
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();

@@ -285,37 +285,71 @@ __global__ void __launch_bounds__(kPmThreads) k_rollout_pm_batch(const RolloutAr
 // A warp per tile of candidates.
 // ---------------------------------------------------------------------------
 
-// Shared-memory layout of a tile: floats between steps (the axes, padded where
-// their count would put the steps of pass 2's lanes on the same banks) and
-// between candidates (the shortest 16-byte row on which the fewest lanes of
-// pass 1, q on candidate q / K and axis q % K, share a bank).
+// Floats between a tile's steps: the axes, padded where their count would put
+// the steps of pass 2's lanes on the same banks.
+constexpr int pm_tile_step(int K) { return K % 8 == 0 ? K + 4 : K; }
+
+// Floats between a tile's candidates: the shortest 16-byte row of T steps on which
+// the fewest lanes of pass 1, q on candidate q / K and axis q % K, share a bank.
+constexpr int pm_tile_conflicts(int K, int row) {
+  int hits[32] = {}, most = 0;
+  for (int q = 0; q < 32; ++q) most = std::max(most, ++hits[(q / K * row + q % K) % 32]);
+  return most;
+}
+constexpr int pm_tile_row(int K, int T) {
+  const int least = (T * pm_tile_step(K) + 3) / 4 * 4;
+  int best = least, fewest = pm_tile_conflicts(K, least);
+  for (int y = least + 4; y < least + 32; y += 4) {
+    const int conflicts = pm_tile_conflicts(K, y);
+    if (conflicts < fewest) {
+      best = y;
+      fewest = conflicts;
+    }
+  }
+  return best;
+}
+
+// Shared-memory layout of a tile of T = 4 << i steps, i = 0 .. 4.  The rows are
+// found by the compiler: searched at every launch they took 20 to 60 us of the
+// host, more than the launch and a small rollout themselves (4 axes, 1384
+// candidates of 44 steps, called one after another: 20.3 us, now 9.7).
 template <int K>
 struct PmTileShape {
-  static constexpr int kStep = K % 8 == 0 ? K + 4 : K;
-  static int conflicts(int row) {
-    int most = 0;
-    for (int b = 0; b < 32; ++b) {
-      int hits = 0;
-      for (int q = 0; q < 32; ++q) hits += (q / K * row + q % K) % 32 == b;
-      most = std::max(most, hits);
-    }
-    return most;
-  }
-  static int row(int T) {
-    const int least = (T * kStep + 3) / 4 * 4;
-    int best = least;
-    for (int y = least; y < least + 32; y += 4)
-      if (conflicts(y) < conflicts(best)) best = y;
-    return best;
-  }
+  static constexpr int kStep = pm_tile_step(K);
+  static constexpr int kLengths = 5;
+  static constexpr int kRow[kLengths] = {pm_tile_row(K, 4), pm_tile_row(K, 8), pm_tile_row(K, 16), pm_tile_row(K, 32),
+                                         pm_tile_row(K, 64)};
   // two buffers of controls, velocity, position and gain of every axis, costs
-  static int floats(int C, int T) { return (C * (2 * row(T) + 3 * K + T + 1) + 3) / 4 * 4; }
+  static constexpr int floats(int C, int i) { return (C * (2 * kRow[i] + 3 * K + (4 << i) + 1) + 3) / 4 * 4; }
 };
+
+// A warp's tile: C candidates, T steps, its row and floats of shared memory; and
+// the threads per block.  About six warps per SM or more before a warp takes a
+// second candidate; up to eight candidates per warp, two beyond 8 axes, whose rows
+// fill the shared memory first.  T up to 64 steps, as far as a tile takes 16 KB.
+// Measured (us a call, replayed from a graph; C and T swept over 1 .. 32 and
+// 8 .. 128): 2 axes, B 512, H 64: C 1 / 2 / 8 at T 64: 5.4 / 5.6 / 7.9 (21 as one
+// candidate per lane); 2 axes, B 8192, H 128: C 1 / 2 / 4 / 8: 29 / 19 / 14 / 14;
+// 12 axes, B 8192, H 256: C 1 / 2 / 4 / 8: 63 / 49 / 56 / 55 (227 as one candidate
+// per lane); 16 axes, B 8192, H 128: C 2, T 32 / 64: 34 / 47.
+struct PmTile {
+  int C, T, row, floats, block;
+};
+template <int K>
+PmTile pm_tile(long long rows) {
+  using Shape = PmTileShape<K>;
+  int C = K > 8 ? 2 : 8, i = Shape::kLengths - 1, block = 128;
+  const long long want = (long long)device_sms() * 6;
+  while (C > 1 && rows / C < want) C >>= 1;
+  while (i > 0 && Shape::floats(C, i) > 4096) --i;
+  while (block > 32 && rows / C * 32 < (long long)block * device_sms()) block >>= 1;
+  return {C, 4 << i, Shape::kRow[i], Shape::floats(C, i), block};
+}
 
 // Candidates r0 .. r0 + C - 1 (those below a.rows) of one instance by one warp;
 // every lane calls it.  pm: in shared memory; sm: this warp's
-// PmTileShape<K>::floats(C, T) floats, 16-byte aligned; row =
-// PmTileShape<K>::row(T); C <= 32, T a multiple of 4.
+// PmTileShape<K>::floats of C and T, 16-byte aligned; row: its kRow; C <= 32, T a
+// multiple of 4.
 // STATES: also writes the states of the one candidate asked for to a.X.
 template <int K, bool STATES>
 __device__ __forceinline__ void rollout_pm_tile(const RolloutArgs& a, const PointMassModel& pm, int r0, int C, int T,

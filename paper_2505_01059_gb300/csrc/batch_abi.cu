@@ -28,7 +28,8 @@ struct BatchGroup {
   int total_rows = 0;
   int block = 128;
   int chunk = 0;              // horizon chunk of staged control loads (0: direct loads)
-  bool stageable = false;     // every member's rows can be staged (see can_stage)
+  bool pieces = false;        // every member's rows are whole 16-byte pieces (see can_stage)
+  bool stageable = false;     // and they are a chain's, whose staging the autotuner decides
   // this group's share of the generation, selection and update launches
   int z_blocks = 0, cand_blocks = 0, local_blocks = 0, upd_threads = 0;
   // members whose graph rows are contracted on the tensor cores (BF16 basis):
@@ -178,6 +179,7 @@ struct mtp_batch {
   cudaEvent_t persist_ev2 = nullptr;
   cudaStream_t group_stream_hi[kMaxGroups] = {};  // high priority: the first launch's generation
   size_t p_warp_bytes[2] = {0, 0};  // shared memory per warp: staged mode, direct mode
+  bool p_pm_direct = false;     // PersistArgs::pm_direct
   int p_blocks[2] = {0, 0};     // resident CTAs per SM: staged mode, direct mode
   cudaEvent_t persist_ev = nullptr;
   double mode_ms[4] = {0, 0, 0, 0};  // the autotuner's iteration time per mode (0: not timed)
@@ -423,9 +425,10 @@ cudaError_t fill_batch(mtp_batch* b, mtp_handle* const* handles, int count, cuda
       row[j + 1] = row[j] + ((h->dm.B + 31) / 32) * 32;  // whole warps per instance
     }
     g.total_rows = row[g.count];
-    g.stageable = g.dyn == MTP_DYN_CHAIN;
+    g.pieces = g.dyn != MTP_DYN_LEGGED;
     for (int j = 0; j < g.count; ++j)
-      g.stageable = g.stageable && can_stage(hv.d_ra[g.first + j], group_key_n(handles[order[g.first + j]]));
+      g.pieces = g.pieces && can_stage(hv.d_ra[g.first + j], group_key_n(handles[order[g.first + j]]));
+    g.stageable = g.pieces && g.dyn == MTP_DYN_CHAIN;
     if (!g.stageable) g.chunk = 0;
     rs += g.count + 1;
   }
@@ -448,6 +451,7 @@ cudaError_t fill_batch(mtp_batch* b, mtp_handle* const* handles, int count, cuda
     std::vector<Entry> ent;
     size_t pm_floats = 0;
     int max_links = 0;
+    b->p_pm_direct = false;
     for (size_t gi = 0; gi < b->groups.size(); ++gi) {
       const BatchGroup& g = b->groups[gi];
       const bool cov = (g.dyn == MTP_DYN_POINTMASS && g.n <= kPersistMaxAxes) ||
@@ -462,8 +466,12 @@ cudaError_t fill_batch(mtp_batch* b, mtp_handle* const* handles, int count, cuda
         const int pos = g.first + j;
         const mtp_handle* h = handles[order[pos]];
         const bool stage = can_stage(hv.d_ra[pos], g.n);
-        if (g.dyn == MTP_DYN_POINTMASS) pm_floats = std::max(pm_floats, persist_pm_floats(g.n));
-        else if (stage) max_links = std::max(max_links, g.n);
+        if (g.dyn == MTP_DYN_POINTMASS) {
+          pm_floats = std::max(pm_floats, persist_pm_floats(g.n));
+          b->p_pm_direct |= !stage;
+        } else if (stage) {
+          max_links = std::max(max_links, g.n);
+        }
         ent.push_back({per_step * h->dm.H, pos, g.dyn | (g.n << 8) | (stage ? 1 << 16 : 0),
                        g.model_first + j, (h->dm.B + 31) / 32});
       }
@@ -523,7 +531,7 @@ cudaError_t fill_batch(mtp_batch* b, mtp_handle* const* handles, int count, cuda
     b->p_total_warps = w;
     b->p_warp_bytes[0] = persist_warp_bytes(pm_floats, max_links);
     b->p_warp_bytes[1] = persist_warp_bytes(pm_floats, 0);
-    for (int k = 0; k < 2; ++k) b->p_blocks[k] = persist_blocks_per_sm(b->p_warp_bytes[k]);
+    for (int k = 0; k < 2; ++k) b->p_blocks[k] = persist_blocks_per_sm(b->p_warp_bytes[k], b->p_pm_direct);
     if (b->p_count > 0 && (b->p_blocks[0] < 1 || b->p_blocks[1] < 1)) return cudaErrorInvalidConfiguration;
   }
   // packing of x0 and u*, in the caller's order
@@ -565,7 +573,7 @@ cudaError_t launch_group(const mtp_batch* b, const BatchGroup& g, int block, int
   const int* rs = t.d_row_start + g.rows_first;
   if (!g.stageable) chunk = 0;
   if (g.dyn == MTP_DYN_POINTMASS)
-    return launch_rollout_pointmass_batch(ra, t.d_pm + g.model_first, rs, g.count, g.total_rows, g.n, block, s);
+    return launch_rollout_pointmass_batch(ra, t.d_pm + g.model_first, rs, g.count, g.total_rows, g.n, block, g.pieces, s);
   if (g.dyn == MTP_DYN_LEGGED)  // fixed 64-thread blocks (shared-memory staging)
     return launch_rollout_legged_batch(ra, t.d_lm + g.model_first, rs, g.count, g.total_rows, g.n, s);
   return launch_rollout_chain_batch(ra, t.d_cm + g.model_first, rs, g.count, g.total_rows, g.n, block,
@@ -595,6 +603,7 @@ PersistArgs persist_args(const mtp_batch* b, bool staged, int part = 0) {
   p.w_base = 0;
   p.warp_bytes = b->p_warp_bytes[staged ? 0 : 1];
   p.staged = staged ? 1 : 0;
+  p.pm_direct = b->p_pm_direct ? 1 : 0;
   if (part == 1) {
     p.count = b->p_split;
     p.total_warps = b->p_split_warps;

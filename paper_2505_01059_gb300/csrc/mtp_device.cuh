@@ -318,6 +318,7 @@ struct PersistArgs {
   int w_base;         // wstart[0]: the first tile of these entries in the batch's numbering
   size_t warp_bytes;  // shared memory per warp: the largest tile
   int staged;         // chain tiles stage their controls where their rows allow it (else direct loads)
+  int pm_direct;      // some point mass's rows do not allow it: they are loaded directly
 };
 // Shared memory per warp: a point mass's tile of `axes` axes, in floats; and
 // all of a warp's, for point-mass tiles of at most pm_floats and staged chain
@@ -327,7 +328,7 @@ size_t persist_warp_bytes(size_t pm_floats, int max_links_staged);
 // Resident 128-thread CTAs per SM of the persistent launch with that much
 // shared memory per warp (0 on error); also sets the launch's shared-memory
 // attribute.
-int persist_blocks_per_sm(size_t warp_bytes);
+int persist_blocks_per_sm(size_t warp_bytes, bool pm_direct);
 cudaError_t launch_rollout_persistent(const PersistArgs& p, int blocks_per_sm, cudaStream_t s);
 // Def. 2 graph rows on the tensor cores (BF16 operands, FP32 sums): whether a
 // generation's graph part goes there (BF16 B-spline, H <= 256, M <= 64,
@@ -370,7 +371,7 @@ cudaError_t launch_candidates_batch(const CandArgs* d_args, const int* d_block_s
                                     int total_blocks, size_t smem, cudaStream_t s);
 cudaError_t launch_rollout_pointmass_batch(const RolloutArgs* d_ra, const PointMassModel* d_pm,
                                            const int* d_row_start, int count, int total_rows,
-                                           int k, int block, cudaStream_t s);
+                                           int k, int block, bool staged, cudaStream_t s);
 cudaError_t launch_rollout_chain_batch(const RolloutArgs* d_ra, const ChainModel* d_cm,
                                        const int* d_row_start, int count, int total_rows,
                                        int links, int block, int chunk, cudaStream_t s);

@@ -47,11 +47,18 @@ namespace {
 
 constexpr int kPersistThreads = 128;
 
-template <int K>
-__device__ __forceinline__ void pm_item(int k, const RolloutArgs& a, const PointMassModel& m, int r0, float* buf) {
+template <int K, bool DIRECT>
+__device__ __forceinline__ void pm_item(int k, bool pieces, const RolloutArgs& a, const PointMassModel& m, int r0,
+                                        float* buf) {
   if constexpr (K <= kPersistMaxAxes) {
-    if (k == K) rollout_pm_lanes<K, PmLane<K>::P, PmLane<K>::T>(a, m, r0, buf);
-    else pm_item<K + 1>(k, a, m, r0, buf);
+    using L = PmLane<K>;
+    if (k == K) {
+      if constexpr (DIRECT)
+        if (!pieces) return rollout_pm_lanes_direct<K, L::P>(a, m, r0);
+      rollout_pm_lanes<K, L::P, L::T>(a, m, r0, buf);
+    } else {
+      pm_item<K + 1, DIRECT>(k, pieces, a, m, r0, buf);
+    }
   }
 }
 
@@ -71,6 +78,10 @@ __device__ __forceinline__ void chain_item(int links, bool staged, const Rollout
   }
 }
 
+// DIRECT: some point mass's rows are not whole 16-byte pieces and are loaded
+// directly.  A kernel of its own: with both forms of every point mass in it, the
+// batch of 256, which has no such rows, took 1.913 ms instead of 1.899.
+template <bool DIRECT>
 __global__ void __launch_bounds__(kPersistThreads, 3) k_rollout_persistent(const PersistArgs p) {
   __shared__ PointMassModel models[kPersistThreads / 32];
   extern __shared__ __align__(16) unsigned char persist_smem[];
@@ -96,7 +107,7 @@ __global__ void __launch_bounds__(kPersistThreads, 3) k_rollout_persistent(const
     const int dim = (code >> 8) & 0xff;
     if ((code & 0xff) == MTP_DYN_POINTMASS) {
       load_pm_model(models[warp], p.pm[model]);
-      pm_item<1>(dim, a, models[warp], r0, buf);
+      pm_item<1, DIRECT>(dim, (code >> 16) != 0, a, models[warp], r0, buf);
     } else {
       const ChainModel cm = p.cm[model];
       // staged only where the instance's rows allow it and the launch asks for it
@@ -125,7 +136,8 @@ size_t persist_warp_bytes(size_t pm_floats, int max_links_staged) {
   return std::max({pm_floats * sizeof(float), chain_bytes_of<1>(max_links_staged), size_t(16)});
 }
 
-int persist_blocks_per_sm(size_t warp_bytes) {
+template <bool DIRECT>
+static int blocks_per_sm_of(size_t warp_bytes) {
   // per device and shared-memory size, computed once: a batch refilled every
   // serving cycle asks again each time
   static std::mutex mu;
@@ -139,15 +151,18 @@ int persist_blocks_per_sm(size_t warp_bytes) {
   // largest tile any batch can have
   const int warps = kPersistThreads / 32;
   const size_t ceiling = persist_warp_bytes(kPmLaneFloats, kPersistMaxLinks) * warps;
-  if (cudaFuncSetAttribute(k_rollout_persistent, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ceiling) !=
+  if (cudaFuncSetAttribute(k_rollout_persistent<DIRECT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ceiling) !=
       cudaSuccess)
     return 0;
   int blocks = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_rollout_persistent, kPersistThreads,
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k_rollout_persistent<DIRECT>, kPersistThreads,
                                                     warp_bytes * warps) != cudaSuccess)
     return 0;
   cache[{dev, warp_bytes}] = blocks;
   return blocks;
+}
+int persist_blocks_per_sm(size_t warp_bytes, bool pm_direct) {
+  return pm_direct ? blocks_per_sm_of<true>(warp_bytes) : blocks_per_sm_of<false>(warp_bytes);
 }
 
 cudaError_t launch_rollout_persistent(const PersistArgs& p, int blocks_per_sm, cudaStream_t s) {
@@ -157,7 +172,9 @@ cudaError_t launch_rollout_persistent(const PersistArgs& p, int blocks_per_sm, c
                                         (p.total_warps + warps_per_block - 1) / warps_per_block));
   cudaError_t e = cudaMemsetAsync(p.head, 0, sizeof(unsigned), s);
   if (e != cudaSuccess) return e;
-  k_rollout_persistent<<<grid, kPersistThreads, p.warp_bytes * warps_per_block, s>>>(p);
+  const size_t smem = p.warp_bytes * warps_per_block;
+  if (p.pm_direct) k_rollout_persistent<true><<<grid, kPersistThreads, smem, s>>>(p);
+  else k_rollout_persistent<false><<<grid, kPersistThreads, smem, s>>>(p);
   return cudaGetLastError();
 }
 

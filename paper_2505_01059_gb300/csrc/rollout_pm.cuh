@@ -252,6 +252,75 @@ __device__ __forceinline__ void rollout_pm_lanes(const RolloutArgs& a, const Poi
   }
 }
 
+// The same for rows that cannot be staged in 16-byte pieces: each lane loads its
+// own row, the next P steps while the current ones' costs are evaluated.  (Copied
+// into shared memory by single floats, such rows took 1.2 to 1.7 times as long as
+// with the direct loads one step ahead that came before: a persistent launch of 600
+// candidates of 7 axes and 101 steps 57 us, 38 so.)
+template <int K, int P>
+__device__ __forceinline__ void rollout_pm_lanes_direct(const RolloutArgs& a, const PointMassModel& pm, int r0) {
+  const int r = r0 + (int)(threadIdx.x & 31);
+  const int H = a.H;
+  const uint32_t iter = a.d_iter ? *a.d_iter : a.iter;
+  const float* const row = a.U + (size_t)min(r, a.rows - 1) * H * K;
+  const int models = (a.dr_mode == MTP_DR_SHARED) ? a.R : 1;
+  const float dt = a.dt;
+  const float w_ctrl = pm.w_ctrl;
+  float total = 0.f;
+  for (int mdl = 0; mdl < models; ++mdl) {
+    float gain[K], v[K], x[K], u[P * K];
+    dr_scales<K>(a, iter, (a.dr_mode == MTP_DR_SHARED) ? (uint32_t)mdl : (uint32_t)(a.row0 + r), gain);
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      gain[k] *= dt;
+      x[k] = a.x0[k];
+      v[k] = a.x0[K + k];
+    }
+    auto load = [&](int t) {
+#pragma unroll
+      for (int q = 0; q < P; ++q) {
+        const float* const s = row + min(t + q, H - 1) * K;
+#pragma unroll
+        for (int k = 0; k < K; ++k) u[q * K + k] = __ldg(s + k);
+      }
+    };
+    load(0);
+    KahanSum J;
+    // step H stands for the terminal cost
+    for (int t = 0; t <= H; t += P) {
+      float p[P][K], uu[P], state[P];
+#pragma unroll
+      for (int q = 0; q < P; ++q) {
+        uu[q] = 0.f;
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+          p[q][k] = x[k];
+          uu[q] = fmaf(u[q * K + k], u[q * K + k], uu[q]);
+          v[k] = fmaf(gain[k], u[q * K + k], v[k]);
+          x[k] = fmaf(dt, v[k], x[k]);
+        }
+      }
+      if (t + P < H) load(t + P);
+      pm_state_costs<K, P>(pm, p, state);
+      if (t + P <= H) {
+#pragma unroll
+        for (int q = 0; q < P; ++q) J.add(fmaf(w_ctrl, uu[q], state[q]), a.kahan);
+      } else {
+#pragma unroll
+        for (int q = 0; q < P; ++q)
+          if (t + q <= H)
+            J.add(t + q < H ? fmaf(w_ctrl, uu[q], state[q]) : __fmul_rn(pm.w_term, state[q]), a.kahan);
+      }
+    }
+    total += J.s;
+  }
+  if (r < a.rows) {
+    float cost = total / (float)models;
+    if (!isfinite(cost)) cost = __int_as_float(0x7f800000);
+    a.cost[r] = cost;
+  }
+}
+
 // The lane body's steps in flight and chunk length: more steps where a position
 // takes few registers, and as long a chunk as kPmLaneFloats hold.
 constexpr int kPmLaneFloats = 4352;
@@ -264,8 +333,8 @@ struct PmLane {
 };
 
 // Many instances: their rows are padded to multiples of 32 (row_start), so a
-// warp's candidates belong to one instance.
-template <int K>
+// warp's candidates belong to one instance.  STAGED: all of them have vector_rows.
+template <int K, bool STAGED>
 __global__ void __launch_bounds__(kPmThreads) k_rollout_pm_batch(const RolloutArgs* __restrict__ ra,
                                                                  const PointMassModel* __restrict__ pm,
                                                                  const int* __restrict__ row_start, int count) {
@@ -278,7 +347,9 @@ __global__ void __launch_bounds__(kPmThreads) k_rollout_pm_batch(const RolloutAr
   load_pm_model(models[warp], pm[i]);
   const RolloutArgs a = ra[i];
   using L = PmLane<K>;
-  rollout_pm_lanes<K, L::P, L::T>(a, models[warp], g - __ldg(row_start + i), pm_smem + warp * L::floats);
+  const int r0 = g - __ldg(row_start + i);
+  if constexpr (STAGED) rollout_pm_lanes<K, L::P, L::T>(a, models[warp], r0, pm_smem + warp * L::floats);
+  else rollout_pm_lanes_direct<K, L::P>(a, models[warp], r0);
 }
 
 // ---------------------------------------------------------------------------

@@ -8,7 +8,16 @@
 namespace mtp {
 namespace {
 
-// Control steps requested ahead of use by the chain rollouts.
+// Threads per block: fill as many SMs as the batch allows (one thread per
+// candidate; small batches get one warp per block).
+inline int rollout_block(int rows) {
+  const int sms = device_sms();
+  int bd = 128;
+  while (bd > 32 && (rows + bd - 1) / bd < sms) bd >>= 1;
+  return bd;
+}
+
+// Control steps requested ahead of use by rollouts that load directly.
 // Measured on GB300 (depths 1 / 2 / 3 / 4): a lone instance, which has one
 // warp per SM sub-partition at most, is fastest at 2 (7-link arm 118 / 105 /
 // 105 / 109 us per step); a batch, where registers set how many warps are

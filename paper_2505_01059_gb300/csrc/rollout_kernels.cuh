@@ -36,15 +36,6 @@ constexpr int kThreads = 128;
 #endif
 constexpr int kSemisepLinks = MTP_SEMISEP_LINKS;
 
-// Threads per block: fill as many SMs as the batch allows (one thread per
-// candidate; small batches get one warp per block).
-inline int rollout_block(int rows) {
-  const int sms = device_sms();
-  int bd = 128;
-  while (bd > 32 && (rows + bd - 1) / bd < sms) bd >>= 1;
-  return bd;
-}
-
 // Dynamic shared memory of a rollout block of `block` threads staging K
 // controls per step T steps at a time (0 for direct loads).
 template <int K, int T>

@@ -9,6 +9,14 @@ template <int K>
 cudaError_t pm_dispatch(const RolloutArgs& a, const PointMassModel& m, cudaStream_t s) {
   if constexpr (K <= kMaxPmAxes) {
     if (a.n == K) {
+      const PmBody body = a.X ? PmBody::kTile : pm_body<K>(a.rows, a.H, can_stage(a, K));
+      if (body != PmBody::kTile) {
+        const int block = body == PmBody::kLanes ? 64 : rollout_block(a.rows), grid = (a.rows + block - 1) / block;
+        if (body == PmBody::kLanes)
+          k_rollout_pm_lanes<K><<<grid, block, block / 32 * PmLane<K>::floats * sizeof(float), s>>>(a, m);
+        else k_rollout_pm_direct<K><<<grid, block, 0, s>>>(a, m);
+        return cudaGetLastError();
+      }
       const PmTile t = pm_tile<K>(a.rows);
       const int tiles = (a.rows + t.C - 1) / t.C, warps = t.block / 32, grid = (tiles + warps - 1) / warps;
       const size_t smem = warps * t.floats * sizeof(float);
@@ -27,7 +35,8 @@ cudaError_t pm_attributes() {
   if constexpr (K <= kMaxPmAxes) {
     cudaError_t e;
     if ((e = cudaFuncSetAttribute(k_rollout_pm<K, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPmSmemMax)) ||
-        (e = cudaFuncSetAttribute(k_rollout_pm<K, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPmSmemMax)))
+        (e = cudaFuncSetAttribute(k_rollout_pm<K, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPmSmemMax)) ||
+        (e = cudaFuncSetAttribute(k_rollout_pm_lanes<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPmSmemMax)))
       return e;
     return pm_attributes<K + 1>();
   } else {

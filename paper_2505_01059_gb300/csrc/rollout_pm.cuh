@@ -4,16 +4,20 @@
 //
 // The double integrator's recursion is two fused multiply-adds per axis and
 // step; nearly all of a step's work is its cost (the distances to the goal and
-// to every obstacle), which nothing of a later step waits for.  Both bodies
-// evaluate several steps' costs at once; they use the same operations in the
-// same order for every value, so a cost does not depend on which one ran.
+// to every obstacle), which nothing of a later step waits for.  The bodies use
+// the same operations in the same order for every value, so a cost does not
+// depend on which one ran (pm_body says which one a lone instance takes, and why).
 //
-// Many candidates (rollout_pm_lanes: batches): a lane walks its candidate's
-// horizon, P steps' costs in flight.  Bound by the issue slots of the distances;
-// one step at a time left fixed latencies in the open (the batch of 256: 2.68 ->
-// 2.43 ms per iteration).
+// Many candidates (rollout_pm_lanes: batches, large lone instances): a lane walks
+// its candidate's horizon, P steps' costs in flight.  Bound by the issue slots of
+// the distances; one step at a time left fixed latencies in the open (the batch of
+// 256: 2.68 -> 2.43 ms per iteration).
 //
-// Few candidates (rollout_pm_tile: a lone instance): a warp takes C candidates
+// Short horizons, and rows that cannot be staged (rollout_pm_direct): the same a
+// step at a time, with nothing through shared memory and the model as constant
+// operands.
+//
+// Few candidates (rollout_pm_tile: lone instances): a warp takes C candidates
 // T steps at a time, and its lanes share each of three passes over the chunk:
 //   1. the C K axes' recursions, one per lane: the control of (candidate, step,
 //      axis) in shared memory is replaced by the position before that step;
@@ -403,16 +407,18 @@ struct PmTileShape {
 // candidate per lane); 2 axes, B 8192, H 128: C 1 / 2 / 4 / 8: 29 / 19 / 14 / 14;
 // 12 axes, B 8192, H 256: C 1 / 2 / 4 / 8: 63 / 49 / 56 / 55 (227 as one candidate
 // per lane); 16 axes, B 8192, H 128: C 2, T 32 / 64: 34 / 47.
+constexpr int pm_tile_most(int K) { return K > 8 ? 2 : 8; }
+constexpr int kPmTileFloats = 4096;
 struct PmTile {
   int C, T, row, floats, block;
 };
 template <int K>
 PmTile pm_tile(long long rows) {
   using Shape = PmTileShape<K>;
-  int C = K > 8 ? 2 : 8, i = Shape::kLengths - 1, block = 128;
+  int C = pm_tile_most(K), i = Shape::kLengths - 1, block = 128;
   const long long want = (long long)device_sms() * 6;
   while (C > 1 && rows / C < want) C >>= 1;
-  while (i > 0 && Shape::floats(C, i) > 4096) --i;
+  while (i > 0 && Shape::floats(C, i) > kPmTileFloats) --i;
   while (block > 32 && rows / C * 32 < (long long)block * device_sms()) block >>= 1;
   return {C, 4 << i, Shape::kRow[i], Shape::floats(C, i), block};
 }
@@ -578,6 +584,124 @@ __global__ void __launch_bounds__(kPmThreads) k_rollout_pm(const __grid_constant
   if (r0 >= a.rows) return;
   load_pm_model(models[warp], pm);
   rollout_pm_tile<K, STATES>(a, models[warp], r0, C, T, row, pm_smem + warp * warp_floats);
+}
+
+// The same, a lane per candidate (rows of whole 16-byte pieces).
+template <int K>
+__global__ void __launch_bounds__(kPmThreads) k_rollout_pm_lanes(const __grid_constant__ RolloutArgs a,
+                                                                 const __grid_constant__ PointMassModel pm) {
+  extern __shared__ __align__(16) float pm_smem[];
+  __shared__ PointMassModel models[kPmThreads / 32];
+  const int warp = threadIdx.x >> 5;
+  const int r0 = (int)(blockIdx.x * blockDim.x + threadIdx.x) & ~31;
+  if (r0 >= a.rows) return;
+  load_pm_model(models[warp], pm);
+  using L = PmLane<K>;
+  rollout_pm_lanes<K, L::P, L::T>(a, models[warp], r0, pm_smem + warp * L::floats);
+}
+
+// The same, a candidate per thread, one step at a time.  Every obstacle slot is
+// evaluated, with no branch: one basic block, so the obstacles' SFU latencies
+// overlap, and every model index is a constant (those past n_obs have radius 0 and
+// add exactly +0).  (Its parameters are not __grid_constant__: that form took up to
+// 20 % longer, 8 axes above all.)
+template <int K>
+__global__ void __launch_bounds__(kPmThreads) k_rollout_pm_direct(const RolloutArgs a, const PointMassModel pm) {
+  const int r = (int)(blockIdx.x * blockDim.x + threadIdx.x);
+  if (r >= a.rows) return;
+  const uint32_t iter = a.d_iter ? *a.d_iter : a.iter;
+  const int models = (a.dr_mode == MTP_DR_SHARED) ? a.R : 1;
+  const float dt = a.dt;
+  auto state_cost = [&](const float (&p)[K]) {
+    float dist2 = 0.f, pen = 0.f;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      const float e = p[k] - pm.target[k];
+      dist2 = fmaf(e, e, dist2);
+    }
+#pragma unroll
+    for (int o = 0; o < MTP_MAX_OBSTACLES; ++o) {
+      float d2 = 0.f;
+#pragma unroll
+      for (int k = 0; k < K; ++k) {
+        const float e = p[k] - pm.obs_c[o][k];
+        d2 = fmaf(e, e, d2);
+      }
+      pen += fmaxf(pm.obs_r[o] - __fmul_rn(d2, rsqrt_normal(fmaxf(d2, kMinNormal))), 0.f);
+    }
+    return fmaf(pm.w_target, dist2, pm.w_obs * pen);
+  };
+  float total = 0.f;
+  for (int mdl = 0; mdl < models; ++mdl) {
+    float gain[K], x[K], v[K];
+    dr_scales<K>(a, iter, (a.dr_mode == MTP_DR_SHARED) ? (uint32_t)mdl : (uint32_t)(a.row0 + r), gain);
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      gain[k] *= dt;
+      x[k] = a.x0[k];
+      v[k] = a.x0[K + k];
+    }
+    KahanSum J;
+    for_each_step<K, kPrefetchAlone, 0>(a.U + (size_t)r * a.H * K, a.H, nullptr, [&](int, const float (&u)[K]) {
+      float uu = 0.f;
+#pragma unroll
+      for (int k = 0; k < K; ++k) uu = fmaf(u[k], u[k], uu);
+      J.add(fmaf(pm.w_ctrl, uu, state_cost(x)), a.kahan);
+#pragma unroll
+      for (int k = 0; k < K; ++k) {
+        v[k] = fmaf(gain[k], u[k], v[k]);
+        x[k] = fmaf(dt, v[k], x[k]);
+      }
+    });
+    J.add(__fmul_rn(pm.w_term, state_cost(x)), a.kahan);
+    total += J.s;
+  }
+  float cost = total / (float)models;
+  if (!isfinite(cost)) cost = __int_as_float(0x7f800000);
+  a.cost[r] = cost;
+}
+
+// Which body a lone instance's costs take.  A tile evaluates more than a lane of
+// its own does and pays for its passes in barriers; what it gains is warps, and
+// loads that are coalesced and ahead of their use.  So: not for horizons of a few
+// steps, and while the tiles are resident at once, in `wave`, or in up to four times
+// as many where a lane's direct loads are at their worst (rows whole cache lines
+// apart, whose lines fall on the same few sets of the L1, and 12 or 16 axes).  Past
+// that many candidates the lanes' own form, staged if the rows can be.  The lines
+// were drawn through 3646 sizes (1 to 16 axes, 500 to 300000 candidates, 8 to 256
+// steps), where this choice is within 5 % of the faster of the tile and the direct
+// form or better, but for a few; us tile / lanes / direct: 7 axes of 33 steps, 4096
+// candidates 8.5 / - / 18.2, 30000 candidates 34.5 / - / 20.5; 12 axes of 64 steps,
+// 4096 candidates 11.9 / 30.5 / 41.7, 32768 candidates 58.9 / 38.6 / 102.9; 2 axes of
+// 9 steps, 8192 candidates 5.7 / - / 4.4.
+enum class PmBody { kTile, kLanes, kDirect };
+
+// Candidates whose full tiles an SM holds at once: blocks of four warps.
+template <int K>
+constexpr int pm_wave_rows() {
+  using Shape = PmTileShape<K>;
+  const int C = pm_tile_most(K);
+  int i = Shape::kLengths - 1;
+  while (i > 0 && Shape::floats(C, i) > kPmTileFloats) --i;
+  const int bytes = 4 * (Shape::floats(C, i) * (int)sizeof(float) + (int)sizeof(PointMassModel)) + 1024;
+  return std::min(16, 228 * 1024 / bytes) * 4 * C;
+}
+
+template <int K>
+PmBody pm_body(long long rows, int H, bool pieces) {
+  const PmBody many = pieces && H >= (K % 4 == 0 ? 20 : 32) && rows >= 118LL * device_sms() ? PmBody::kLanes : PmBody::kDirect;
+  if (H < (K > 4 ? 12 : 16)) return many;
+  // percent of a wave up to which the tile is taken
+  const bool worst = (K > 8 && K % 4 == 0) || (long long)H * K % 32 == 0;
+  int most;
+  if (H < 32) most = K > 8 && K % 4 == 0 && H >= 20 ? 170 : 90 * H / 32;
+  else if (worst && (K > 4 || H >= 48)) most = 400;
+  else if (H >= 200) most = 300;
+  else if (pieces && H >= 48) most = 200;
+  else if (H >= 96) most = 140;
+  else most = 100;
+  if (K == 1) most = std::min(most, H < 48 ? 50 : 100);
+  return 100 * rows <= (long long)most * pm_wave_rows<K>() * device_sms() ? PmBody::kTile : many;
 }
 
 }  // namespace

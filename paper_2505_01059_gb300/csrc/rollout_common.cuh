@@ -75,9 +75,11 @@ __device__ __forceinline__ float round_nearest(float x) {
 
 // sin and cos of an absolute link angle: Cody-Waite reduction of x by 2 pi
 // (a two-term split of 2 pi) to [-pi, pi], then the SFU sine / cosine, whose
-// absolute error on that interval is about 4e-7.
+// absolute error on that interval is about 4e-7.  SFU: the whole turns by rintf.
+template <bool SFU = false>
 __device__ __forceinline__ void sincos_reduced(float x, float* s, float* c) {
-  const float k = round_nearest(__fmul_rn(x, 0.15915494309189535f));
+  const float turns = __fmul_rn(x, 0.15915494309189535f);
+  const float k = SFU ? rintf(turns) : round_nearest(turns);
   float r = fmaf(-k, 6.28318548202514648f, x);
   r = fmaf(-k, -1.7484556e-07f, r);
   __sincosf(r, s, c);

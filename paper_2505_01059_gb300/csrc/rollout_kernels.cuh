@@ -36,6 +36,15 @@ constexpr int kThreads = 128;
 #endif
 constexpr int kSemisepLinks = MTP_SEMISEP_LINKS;
 
+// Whether a chain of NL links takes its angles' whole turns by rintf (the same
+// value).  The shorter way off the SFU is the faster one for most link counts (lone:
+// 3 links 24.4 against 25.5 us, 9 links 85.5 / 87.1, 12 links 98.4 / 101.8, 128
+// steps) but not where the step is one short chain of instructions (batches of one
+// link, 101 steps: 22.7 against 13.1 us) and not for five links alone, 128 steps of
+// which took 46.2 against 36.4 us (in batches 44 / 45).
+template <int NL, int PF>
+constexpr bool kSfuTurns = NL == 1 || (NL == 5 && PF == kPrefetchAlone);
+
 // Dynamic shared memory of a rollout block of `block` threads staging K
 // controls per step T steps at a time (0 for direct loads).
 template <int K, int T>
@@ -121,7 +130,7 @@ __device__ __forceinline__ void rollout_chain_body(const RolloutArgs& a, const C
 #pragma unroll
       for (int j = 0; j < NL; ++j) {
         tau[j] = u[j];
-        sincos_reduced(phi[j], &s[j], &c[j]);
+        sincos_reduced<kSfuTurns<NL, PF>>(phi[j], &s[j], &c[j]);
       }
       // stage cost c(x_t, u_t): reach error of the tip and torque penalty
       {
@@ -286,7 +295,7 @@ __device__ __forceinline__ void rollout_chain_body(const RolloutArgs& a, const C
     {
       float c[NL], s[NL], x, y;
 #pragma unroll
-      for (int j = 0; j < NL; ++j) sincos_reduced(phi[j], &s[j], &c[j]);
+      for (int j = 0; j < NL; ++j) sincos_reduced<kSfuTurns<NL, PF>>(phi[j], &s[j], &c[j]);
       chain_tip<NL>(len, c, s, x, y);
       const float ex = x - cm.target[0], ey = y - cm.target[1];
       J.add(cm.w_term * cm.w_target * fmaf(ex, ex, ey * ey), a.kahan);

@@ -41,20 +41,9 @@ cudaError_t chain_attributes() {
 
 cudaError_t init_rollout_chain_attributes() { return chain_attributes<1>(); }
 
-// Direct loads two steps ahead, or staged ones?  A lone warp per SM sub-partition
-// waits for its longest chain of instructions either way, and which form's code
-// is the shorter one was measured (us, direct / staged, 128 steps of 4096
-// candidates or 64 of 2048): 3 links 32.0 / 25.7, 4 links 30.6 / 35.2, 5 links
-// 27 / 34 (2048, 100 steps), 7 links 50 / 58, 9 links 85 / 90, 10 links 53 / 47, 12
-// links 54 / 53.  Once several warps share a sub-partition, staged: its loads are
-// coalesced (16384 candidates, 7 links: 65 / 59).
-static bool stages_alone(int links, int rows) {
-  return links <= 3 || links >= 10 || rows > 96 * device_sms();
-}
-
 cudaError_t launch_rollout_chain(const RolloutArgs& a, const ChainModel& m, int links, cudaStream_t s) {
   if (a.rows <= 0) return cudaSuccess;
-  return chain_dispatch<1>(a, m, links, can_stage(a, links) && stages_alone(links, a.rows), s);
+  return chain_dispatch<1>(a, m, links, can_stage(a, links) && stages_alone(links, a.H, a.rows), s);
 }
 
 int rollout_blocks(int rows) {

@@ -45,6 +45,23 @@ constexpr int kSemisepLinks = MTP_SEMISEP_LINKS;
 template <int NL, int PF>
 constexpr bool kSfuTurns = NL == 1 || (NL == 5 && PF == kPrefetchAlone);
 
+// Direct loads two steps ahead, or staged ones?  Alone a warp waits for its longest
+// chain of instructions either way, and which form's code is the shorter one differs
+// by link count; the direct loads get worse where the rows are whole cache lines
+// apart, whose lines fall on the same few sets of the L1, the more so the more warps
+// share an SM.  Staged over direct time, 32 to 256 steps, by link count:
+//   rows of whole lines, up to 8192 candidates: 1 0.97, 2 0.87, 3 0.77, 4 1.09, 5
+//   1.16, 6 0.93, 7 1.09, 8 0.77, 9 1.02, 10 0.82, 11 0.89, 12 0.90; 16384 and 40000:
+//   0.5 to 0.9 for all;
+//   other rows, up to 8192 candidates: 2 0.98, 3 0.83, 4 1.12, 5 1.22, 6 0.98, 7
+//   1.11, 9 1.13, 10 0.92, 11 1.02, 12 0.97; 40000: 0.9 to 1.09, and shared models
+//   of one link 1.09 on any rows.
+inline bool stages_alone(int links, int H, int rows) {
+  const bool lines = (long long)H * links % 32 == 0;
+  if (links == 1 || links == 4 || links == 5 || links == 7 || links == 9) return lines && rows > 96 * device_sms();
+  return lines || (links != 11 && rows <= 192 * device_sms());
+}
+
 // Dynamic shared memory of a rollout block of `block` threads staging K
 // controls per step T steps at a time (0 for direct loads).
 template <int K, int T>

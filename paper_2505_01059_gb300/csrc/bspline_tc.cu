@@ -104,30 +104,6 @@ __host__ __device__ constexpr int tc_paths_per_tile(int n) {
   return 4 * tc_paths_per_warp(n);
 }
 
-// Waits for the MMA's commit, bounded by 2 s of global time; backs off
-// between polls so that the waiting warps leave the issue slots to the
-// co-resident CTAs' epilogues.
-__device__ __forceinline__ bool mbar_wait_bounded_tc(uint64_t* bar, uint32_t parity) {
-  const unsigned addr = smem_u32(bar);
-  uint64_t t_start = 0;
-  for (int spin = 0;; ++spin) {
-    uint32_t done;
-    asm volatile(
-        "{\n .reg .pred p;\n"
-        " mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-        " selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(done)
-        : "r"(addr), "r"(parity)
-        : "memory");
-    if (done) return true;
-    uint64_t now;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
-    if (spin == 0) t_start = now;
-    else if (now - t_start > 2000000000ull) return false;
-    if (spin >= 4) __nanosleep(64);
-  }
-}
-
 __host__ __device__ __forceinline__ bool graph_staged(const CandArgs& a) {
   return a.C_in == nullptr && a.dm.M * a.dm.N * a.dm.n <= kZsMax;
 }
@@ -257,7 +233,7 @@ __device__ __forceinline__ bool tc_tile(TcSmem& S, const CandArgs& a, const TcPl
                      smem_u32(&S.mma_bar))
                  : "memory");
   }
-  const bool ok = mbar_wait_bounded_tc(&S.mma_bar, phase);
+  const bool ok = mbar_wait_bounded(&S.mma_bar, phase);
   phase ^= 1u;
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   if (!__syncthreads_and(ok)) return false;
@@ -362,7 +338,7 @@ __device__ void tc_begin(TcSmem& S) {
 // for the MMA still in flight.
 __device__ void tc_end(TcSmem& S, bool failed, uint32_t phase, uint32_t* status) {
   if (failed) {
-    mbar_wait_bounded_tc(&S.mma_bar, phase ^ 1u);
+    mbar_wait_bounded(&S.mma_bar, phase ^ 1u);
     if (threadIdx.x == 0 && status) atomicOr(status, kStatusTcTimeout);
   }
   __syncthreads();

@@ -196,6 +196,31 @@ struct RolloutArgs {
   int32_t kahan;
 };
 
+// Bounded mbarrier wait (the contraction's wait for its MMA, and the self-test's):
+// try_wait on the phase with the given parity for at most limit_ns of the global
+// timer, then give up (false).  It backs off between polls, so that the waiting
+// warps leave the issue slots to the co-resident CTAs' epilogues.
+__device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity, uint64_t limit_ns = 2000000000ull) {
+  const unsigned addr = (unsigned)__cvta_generic_to_shared(bar);
+  uint64_t t_start = 0;
+  for (int spin = 0;; ++spin) {
+    uint32_t done;
+    asm volatile(
+        "{\n .reg .pred p;\n"
+        " mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+        " selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(done)
+        : "r"(addr), "r"(parity)
+        : "memory");
+    if (done) return true;
+    uint64_t now;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
+    if (spin == 0) t_start = now;
+    else if (now - t_start > limit_ns) return false;
+    if (spin >= 4) __nanosleep(64);
+  }
+}
+
 // Bit of a handle's device status word, set when a bounded wait gave up: the
 // tensor-core contraction's wait for its MMA (those graph rows are not written).
 constexpr uint32_t kStatusTcTimeout = 2u;

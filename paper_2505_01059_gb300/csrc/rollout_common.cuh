@@ -94,30 +94,6 @@ __device__ __forceinline__ void copy_async_f32(float* smem_dst, const float* gme
 __device__ __forceinline__ void copy_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void copy_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
-// Bounded mbarrier wait: try_wait on the phase with the given parity for at
-// most limit_ns of the global timer (about two seconds by default), then
-// give up (returns false).
-__device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity,
-                                                  uint64_t limit_ns = 2000000000ull) {
-  const unsigned addr = (unsigned)__cvta_generic_to_shared(bar);
-  uint64_t t_start = 0;
-  for (int spin = 0;; ++spin) {
-    uint32_t done;
-    asm volatile(
-        "{\n .reg .pred p;\n"
-        " mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-        " selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(done)
-        : "r"(addr), "r"(parity)
-        : "memory");
-    if (done) return true;
-    uint64_t now;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
-    if (spin == 0) t_start = now;
-    else if (now - t_start > limit_ns) return false;
-  }
-}
-
 // ---------------------------------------------------------------------------
 // Staged control rows.  A rollout thread reads its candidate's controls one
 // step after another; a warp's 32 lanes read 32 different rows, H * n floats

@@ -5,7 +5,7 @@
 // returns, and the context stays usable.
 #include <chrono>
 
-#include "rollout_common.cuh"
+#include "mtp_device.cuh"
 
 namespace mtp {
 namespace {

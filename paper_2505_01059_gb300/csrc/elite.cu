@@ -614,53 +614,44 @@ __device__ __forceinline__ void update_body(const UpdateArgs& a, int gt, int thr
       p2[j] = 0.0;
     }
     // virtual lane v = sub + G j takes elites v, v + 32, ... in that order.
-    // With few virtual lanes per thread, R rounds of 32 elites are gathered
-    // at once: first all their indices, then all their rows' values and
-    // weights, so a pass over the elites waits for two dependent loads
-    // rather than two per round.  With many, the P gathers of one round are
-    // already independent and issued together (R = 1).
+    // With a whole warp per element, R rounds of 32 elites are gathered at
+    // once: first all their indices, then all their rows' values and weights,
+    // so a pass over the elites waits for two dependent loads rather than two
+    // per round.  With several virtual lanes per thread, the P gathers of one
+    // round are already independent and issued together.
     auto rounds = [&](auto RR) {
       constexpr int R = decltype(RR)::value;
       for (int k0 = 0; k0 < a.E; k0 += 32 * R) {
-        int idx[R][P];
+        int idx[R];
 #pragma unroll
-        for (int r = 0; r < R; ++r)
+        for (int r = 0; r < R; ++r) {
+          const int k = k0 + 32 * r + sub;
+          idx[r] = k < a.E ? __ldg(a.elite + k) : 0;
+        }
+        float uv[R];
+        double wv[R];
 #pragma unroll
-          for (int j = 0; j < P; ++j) {
-            const int k = k0 + 32 * r + sub + G * j;
-            idx[r][j] = k < a.E ? __ldg(a.elite + k) : 0;
+        for (int r = 0; r < R; ++r) {
+          const int k = k0 + 32 * r + sub;
+          uv[r] = k < a.E ? __ldg(a.U + (size_t)idx[r] * Hn + e) : 0.f;
+          wv[r] = (k < a.E && !cem) ? a.weight[k] : 1.0;
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          const int k = k0 + 32 * r + sub;
+          if (k < a.E) {
+            const double d = (double)uv[r] - c;
+            const double wd = cem ? d : wv[r] * d;
+            p1[0] = p1[0] + wd;
+            p2[0] = fma(wd, d, p2[0]);
           }
-        float uv[R][P];
-        double wv[R][P];
-#pragma unroll
-        for (int r = 0; r < R; ++r)
-#pragma unroll
-          for (int j = 0; j < P; ++j) {
-            const int k = k0 + 32 * r + sub + G * j;
-            uv[r][j] = k < a.E ? __ldg(a.U + (size_t)idx[r][j] * Hn + e) : 0.f;
-            wv[r][j] = (k < a.E && !cem) ? a.weight[k] : 1.0;
-          }
-#pragma unroll
-        for (int r = 0; r < R; ++r)
-#pragma unroll
-          for (int j = 0; j < P; ++j) {
-            const int k = k0 + 32 * r + sub + G * j;
-            if (k < a.E) {
-              const double d = (double)uv[r][j] - c;
-              const double wd = cem ? d : wv[r][j] * d;
-              p1[j] = p1[j] + wd;
-              p2[j] = fma(wd, d, p2[j]);
-            }
-          }
+        }
       }
     };
-    constexpr int R = P == 1 ? kUpdRounds : (P == 2 ? kUpdRounds / 2 : 1);
     if (valid) {
       if constexpr (P == 1) {
         if (a.E > 64) rounds(Rounds<kUpdRoundsMany>{});
-        else rounds(Rounds<R>{});
-      } else if constexpr (R > 1) {
-        rounds(Rounds<R>{});
+        else rounds(Rounds<kUpdRounds>{});
       } else {
         for (int k0 = 0; k0 < a.E; k0 += 32) {
 #pragma unroll
@@ -865,9 +856,8 @@ cudaError_t launch_select(const SelectArgs& a, cudaStream_t s) {
 
 // Two-stage selection plan for B candidates and E elites: the chunk length
 // and chunk count, or chunks = 0 when one block selects them (its keys fit
-// its shared memory and B is at most kOneBlockMax).  Chunks are as long as
-// one block's shared memory allows, and their E-pair outputs must fit the
-// merging block; infeasible sizes return chunks = -1.
+// its shared memory and B is at most kOneBlockMax).  The chunks' E-pair outputs
+// must fit the merging block; infeasible sizes return chunks = -1.
 void select_plan(int B, int E, int* chunk, int* chunks) {
   *chunk = B;
   *chunks = 0;

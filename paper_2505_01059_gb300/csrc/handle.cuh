@@ -49,6 +49,7 @@ struct mtp_handle {
   int prep_grid = 0;          // blocks of k_prepare: one per SM it may take
   int prep_spb = 1;           // graph paths per pass of a k_prepare block
   size_t prep_smem = 0;       // dynamic shared memory of a k_prepare block (a whole SM)
+  bool generated = false;     // mtp_generate_candidates has been called (it makes a side stream from then on)
   cudaStream_t side = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   float* cost = nullptr;

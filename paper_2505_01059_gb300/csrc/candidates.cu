@@ -178,72 +178,110 @@ struct Int {
   static constexpr int value = V;
 };
 
+// Which graph rows a kernel's code makes, so that each is compiled with the
+// registers its own rows need: all of them, or (k_candidates) the heavy ones or the
+// others (heavy_rows).
+enum GraphCode { kGraphAll, kGraphHeavy, kGraphLight };
+
+// Rows of whole 16-byte pieces, in a 16-byte aligned tensor.
+__host__ __device__ __forceinline__ bool vector_graph_rows(const Dims& d, const float* out) {
+  return ((d.H * d.n) & 3) == 0 && (reinterpret_cast<uintptr_t>(out) & 15) == 0;
+}
+
 // Clamped stores of nb consecutive interpolated rows, u = f(path, t, i),
-// coalesced over (t, i).  Four elements per thread and store where the rows are
-// whole 16-byte pieces: a thread count that is a multiple of n / gcd(4, n)
-// makes every stride whole steps, so a thread's four dimensions, their bounds
-// and their steps past the first are fixed, and only (path, t) is carried along.
+// coalesced over (t, i).  A thread count that is a multiple of n (or, four
+// elements at a time, of n / gcd(4, n)) makes every stride whole steps, so a
+// thread's dimensions, their bounds and their steps past the first are fixed, and
+// only (path, t) is carried along.  Four elements per thread and store where the
+// rows are whole 16-byte pieces.
 // (With one element per thread and store, its position stepped and its bounds
 // read for each, and the Akima coefficients made row by row, the batch of 256
 // took 2.22 ms per iteration, now 2.09, the 7-link arm's generation 14.3 us, now
 // 10.7.)
 template <class F>
-__device__ __forceinline__ void store_rows(const CandArgs& a, float* __restrict__ out, int nb, const float* box_lo,
-                                           const float* box_hi, F f) {
+__device__ __forceinline__ void store_rows_by_four(const CandArgs& a, float* __restrict__ out, int nb,
+                                                   const float* box_lo, const float* box_hi, F f) {
   const int H = a.dm.H, n = a.dm.n, Hn = H * n;
   const int total = nb * Hn;
-  if ((Hn & 3) == 0 && (reinterpret_cast<uintptr_t>(out) & 15) == 0) {
-    const int unit = n & 3 ? (n & 1 ? n : n / 2) : n / 4;
-    const int threads = (int)blockDim.x / unit * unit;
-    if ((int)threadIdx.x >= threads) return;
-    int e = 4 * threadIdx.x;
-    int sp = e / Hn, t = (e - sp * Hn) / n, i = e - sp * Hn - t * n;
-    int dim[4], later[4];
-    float lo[4], hi[4];
+  const int unit = n & 3 ? (n & 1 ? n : n / 2) : n / 4;
+  const int threads = (int)blockDim.x / unit * unit;
+  if ((int)threadIdx.x >= threads) return;
+  int e = 4 * threadIdx.x;
+  int sp = e / Hn, t = (e - sp * Hn) / n, i = e - sp * Hn - t * n;
+  int dim[4], later[4];
+  float lo[4], hi[4];
 #pragma unroll
-    for (int w = 0, d = 0; w < 4; ++w) {
-      dim[w] = i;
-      later[w] = d;
-      lo[w] = box_lo[i];
-      hi[w] = box_hi[i];
-      if (++i == n) {
-        i = 0;
-        ++d;
-      }
+  for (int w = 0, d = 0; w < 4; ++w) {
+    dim[w] = i;
+    later[w] = d;
+    lo[w] = box_lo[i];
+    hi[w] = box_hi[i];
+    if (++i == n) {
+      i = 0;
+      ++d;
     }
-    const int stride = 4 * threads, ds = stride / Hn, dt = (stride - ds * Hn) / n;
-    for (; e < total; e += stride) {
-      float o[4];
-#pragma unroll
-      for (int w = 0; w < 4; ++w) o[w] = clamp_box(f(sp, t + later[w], dim[w]), lo[w], hi[w]);
-      *reinterpret_cast<float4*>(out + e) = make_float4(o[0], o[1], o[2], o[3]);
-      sp += ds;
-      t += dt;
-      if (t >= H) {
-        t -= H;
-        ++sp;
-      }
-    }
-    return;
   }
-  int e = threadIdx.x;
-  int sp = e / Hn, rem = e - sp * Hn;
-  int t = rem / n, i = rem - t * n;
-  const int ds = blockDim.x / Hn, drem = blockDim.x - ds * Hn;
-  const int dt = drem / n, di = drem - dt * n;
-  for (; e < total; e += blockDim.x) {
-    out[e] = clamp_box(f(sp, t, i), box_lo[i], box_hi[i]);
+  const int stride = 4 * threads, ds = stride / Hn, dt = (stride - ds * Hn) / n;
+  for (; e < total; e += stride) {
+    float o[4];
+#pragma unroll
+    for (int w = 0; w < 4; ++w) o[w] = clamp_box(f(sp, t + later[w], dim[w]), lo[w], hi[w]);
+    *reinterpret_cast<float4*>(out + e) = make_float4(o[0], o[1], o[2], o[3]);
     sp += ds;
     t += dt;
-    i += di;
-    if (i >= n) {
-      i -= n;
-      ++t;
-    }
     if (t >= H) {
       t -= H;
       ++sp;
     }
+  }
+}
+
+template <class F>
+__device__ __forceinline__ void store_rows_by_one(const CandArgs& a, float* __restrict__ out, int nb,
+                                                  const float* box_lo, const float* box_hi, F f) {
+  const int H = a.dm.H, n = a.dm.n, Hn = H * n;
+  const int total = nb * Hn;
+  const int threads = (int)blockDim.x / n * n;
+  if ((int)threadIdx.x >= threads) return;
+  int e = threadIdx.x;
+  int sp = e / Hn, t = (e - sp * Hn) / n;
+  const int i = e - sp * Hn - t * n;
+  const float lo = box_lo[i], hi = box_hi[i];
+  const int ds = threads / Hn, dt = (threads - ds * Hn) / n;
+  for (; e < total; e += threads) {
+    out[e] = clamp_box(f(sp, t, i), lo, hi);
+    sp += ds;
+    t += dt;
+    if (t >= H) {
+      t -= H;
+      ++sp;
+    }
+  }
+}
+
+// Rows that are Akima's of 3 dimensions or more, or the B-spline's of 4 or more in
+// whole 16-byte pieces: their kernel takes 56 registers and four blocks of an SM, the
+// other rows' 48 and five.  All rows in one kernel with four / five blocks per SM, and
+// each in its own (us): 20000 straight rows of 31 x 15 48.8 / 38.6 / 38.5, 20000
+// B-spline rows of 31 x 15 41.6 / 34.1 / 34.0, 8513 Akima rows of 319 x 16 59.4 / 65.8 /
+// 59.4, 2000 B-spline rows of 65 x 16 15.3 / 18.7 / 15.8.  (Four B-spline elements of
+// few dimensions lie in several steps and share no window: 20000 rows of 100 x 2 four at a
+// time 23.8, one at a time 16.8.)
+__host__ __device__ __forceinline__ bool heavy_rows(int interp, const Dims& d, const float* out) {
+  return interp == MTP_INTERP_AKIMA ? d.n >= 3 : interp == MTP_INTERP_BSPLINE && d.n >= 4 && vector_graph_rows(d, out);
+}
+
+template <int CODE, int KIND, class F>
+__device__ __forceinline__ void store_rows(const CandArgs& a, float* __restrict__ out, int nb, const float* box_lo,
+                                           const float* box_hi, F f) {
+  if constexpr (CODE == kGraphHeavy && KIND == MTP_INTERP_BSPLINE) {
+    store_rows_by_four(a, out, nb, box_lo, box_hi, f);
+  } else if constexpr (CODE == kGraphLight && KIND != MTP_INTERP_LINEAR) {
+    store_rows_by_one(a, out, nb, box_lo, box_hi, f);
+  } else if constexpr (CODE != kGraphHeavy || KIND == MTP_INTERP_AKIMA) {
+    if (vector_graph_rows(a.dm, out) && (KIND == MTP_INTERP_LINEAR || heavy_rows(KIND, a.dm, out)))
+      store_rows_by_four(a, out, nb, box_lo, box_hi, f);
+    else store_rows_by_one(a, out, nb, box_lo, box_hi, f);
   }
 }
 
@@ -252,6 +290,7 @@ __device__ __forceinline__ void store_rows(const CandArgs& a, float* __restrict_
 // global memory) into C (shared memory, followed by the Akima scratch), and
 // the interpolated, clamped rows.  Every path is computed on its own, so the
 // grouping of paths into blocks does not change any value.
+template <int CODE>
 __device__ __forceinline__ void graph_paths_body(const CandArgs& a, const float* Zs, float* C,
                                                  int bid, uint32_t iter, const float* box_lo,
                                                  const float* box_hi) {
@@ -342,7 +381,7 @@ __device__ __forceinline__ void graph_paths_body(const CandArgs& a, const float*
   if (a.interp == MTP_INTERP_BSPLINE) {
     // Def. 2: sum over the (p+1)-wide non-zero window of basis row t.
     auto bspline = [&](auto D) {
-      store_rows(a, out, nb, box_lo, box_hi, [&](int sp, int t, int i) {
+      store_rows<CODE, MTP_INTERP_BSPLINE>(a, out, nb, box_lo, box_hi, [&](int sp, int t, int i) {
         constexpr int deg = decltype(D)::value;
         const int f = bfirst[t];
         const float* brow = basis + (size_t)t * M;
@@ -368,13 +407,13 @@ __device__ __forceinline__ void graph_paths_body(const CandArgs& a, const float*
     }
   } else if (a.interp == MTP_INTERP_AKIMA) {
     const int K1 = M - 1;
-    store_rows(a, out, nb, box_lo, box_hi, [&](int sp, int t, int i) {
+    store_rows<CODE, MTP_INTERP_AKIMA>(a, out, nb, box_lo, box_hi, [&](int sp, int t, int i) {
       const float2 pc = piece[t];
       const float4 cf = coef[(sp * K1 + __float_as_int(pc.x)) * n + i];
       return fmaf(fmaf(fmaf(cf.w, pc.y, cf.z), pc.y, cf.y), pc.y, cf.x);
     });
   } else {
-    store_rows(a, out, nb, box_lo, box_hi, [&](int sp, int t, int i) {
+    store_rows<CODE, MTP_INTERP_LINEAR>(a, out, nb, box_lo, box_hi, [&](int sp, int t, int i) {
       const float2 pc = piece[t];
       const int k = __float_as_int(pc.x);
       const float w = fminf(pc.y * inv_h_t, 1.f);
@@ -385,6 +424,7 @@ __device__ __forceinline__ void graph_paths_body(const CandArgs& a, const float*
 }
 
 // Graph block `bid` of one planning problem.
+template <int CODE>
 __device__ __forceinline__ void graph_block_body(const CandArgs& a, float* smem, int bid) {
   __shared__ float box_lo[MTP_MAX_CTRL], box_hi[MTP_MAX_CTRL];
   stage_box(a, box_lo, box_hi);
@@ -397,12 +437,13 @@ __device__ __forceinline__ void graph_block_body(const CandArgs& a, float* smem,
     __syncthreads();
     Zs = Z;
   }
-  graph_paths_body(a, Zs, C, bid, iter, box_lo, box_hi);
+  graph_paths_body<CODE>(a, Zs, C, bid, iter, box_lo, box_hi);
 }
 
-__global__ void __launch_bounds__(kThreads, 4) k_candidates(const CandArgs a) {
+template <int CODE>
+__global__ void __launch_bounds__(kThreads, CODE == kGraphHeavy ? 4 : 5) k_candidates(const CandArgs a) {
   extern __shared__ __align__(16) float smem[];
-  if ((int)blockIdx.x < a.graph_blocks) graph_block_body(a, smem, blockIdx.x);
+  if ((int)blockIdx.x < a.graph_blocks) graph_block_body<CODE>(a, smem, blockIdx.x);
   else local_rows_body<kLocalFull>(a, (int)blockIdx.x - a.graph_blocks, (int)gridDim.x - a.graph_blocks);
 }
 
@@ -425,7 +466,7 @@ __global__ void __launch_bounds__(kThreads) k_candidates_batch(const CandArgs* _
   int* dst = reinterpret_cast<int*>(&sa);
   for (int w = threadIdx.x; w < (int)(sizeof(CandArgs) / sizeof(int)); w += blockDim.x) dst[w] = src[w];
   __syncthreads();
-  graph_block_body(sa, smem, blk - block_start[lo]);
+  graph_block_body<kGraphAll>(sa, smem, blk - block_start[lo]);
 }
 
 // Local rows of many planning problems (no shared memory, so the blocks
@@ -510,7 +551,7 @@ __global__ void __launch_bounds__(kPrepThreads, 1) k_prepare(const CandArgs a) {
     float* C = Z + graph_floats(a.dm);
     for (int vb = blockIdx.x; vb < a.graph_blocks; vb += gridDim.x) {
       __syncthreads();  // Z complete; the previous paths' scratch no longer read
-      graph_paths_body(a, Z, C, vb, iter, box_lo, box_hi);
+      graph_paths_body<kGraphAll>(a, Z, C, vb, iter, box_lo, box_hi);
     }
   }
   if (a.U_local && a.local_rows > 0) local_rows_body<kLocalNoise>(a, blockIdx.x, gridDim.x);
@@ -584,11 +625,12 @@ size_t candidates_smem_bytes(const CandArgs& a) {
 // Opt in to large dynamic shared memory on the current device (called by
 // mtp_create, outside any stream capture).
 cudaError_t init_candidate_attributes() {
-  cudaError_t e = cudaFuncSetAttribute(k_candidates, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       200 * 1024);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(k_candidates_batch, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              200 * 1024);
+  for (const void* k : {(const void*)k_candidates<kGraphHeavy>, (const void*)k_candidates<kGraphLight>,
+                        (const void*)k_candidates_batch}) {
+    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 cudaError_t launch_candidates_batch(const CandArgs* d_args, const int* d_block_start, int count,
@@ -601,7 +643,9 @@ cudaError_t launch_candidates_batch(const CandArgs* d_args, const int* d_block_s
 cudaError_t launch_candidates(const CandArgs& a, int local_blocks, cudaStream_t s) {
   const int grid = a.graph_blocks + local_blocks;
   if (grid <= 0) return cudaSuccess;
-  k_candidates<<<grid, kThreads, candidates_smem_bytes(a), s>>>(a);
+  const bool heavy = a.graph_blocks <= 0 || heavy_rows(a.interp, a.dm, a.U_graph);  // local rows alone: 62 us heavy, 64.5 light (16384 of 256 x 15, beta 0.3)
+  if (heavy) k_candidates<kGraphHeavy><<<grid, kThreads, candidates_smem_bytes(a), s>>>(a);
+  else k_candidates<kGraphLight><<<grid, kThreads, candidates_smem_bytes(a), s>>>(a);
   return cudaGetLastError();
 }
 

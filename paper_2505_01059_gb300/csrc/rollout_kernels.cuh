@@ -41,9 +41,13 @@ constexpr int kSemisepLinks = MTP_SEMISEP_LINKS;
 // 3 links 24.4 against 25.5 us, 9 links 85.5 / 87.1, 12 links 98.4 / 101.8, 128
 // steps) but not where the step is one short chain of instructions (batches of one
 // link, 101 steps: 22.7 against 13.1 us) and not for five links alone, 128 steps of
-// which took 46.2 against 36.4 us (in batches 44 / 45).
+// which took 46.2 against 36.4 us (in batches 44 / 45).  Nor in direct rollouts of
+// so many lone candidates that the issue slots bound them (turns_by_sfu): 40000 of
+// 36 steps, off the SFU over on it, 2 1.02, 6 1.02, 9 1.02, 10 1.02, 12 1.04, 4, 7, 8
+// and 11 links 1.00 to 1.01; 16384 of 36: 0.96 to 1.00.
 template <int NL, int PF>
 constexpr bool kSfuTurns = NL == 1 || (NL == 5 && PF == kPrefetchAlone);
+inline bool turns_by_sfu(int rows) { return rows > 192 * device_sms(); }
 
 // Direct loads two steps ahead, or staged ones?  Alone a warp waits for its longest
 // chain of instructions either way, and which form's code is the shorter one differs
@@ -56,10 +60,15 @@ constexpr bool kSfuTurns = NL == 1 || (NL == 5 && PF == kPrefetchAlone);
 //   other rows, up to 8192 candidates: 2 0.98, 3 0.83, 4 1.12, 5 1.22, 6 0.98, 7
 //   1.11, 9 1.13, 10 0.92, 11 1.02, 12 0.97; 40000: 0.9 to 1.09, and shared models
 //   of one link 1.09 on any rows.
-inline bool stages_alone(int links, int H, int rows) {
+// Shared models walk the same rows again, which direct loads then find in the L1.
+// Staged over direct time with four of them, other rows, 24 to 100 steps: 32 to 8192
+// candidates, 2 links 0.99 to 1.02, 3 0.94 to 1.00, 6 1.03 to 1.06, 8 0.94 to 1.01, 10
+// 0.98 to 1.07, 12 1.04 to 1.11; 16384: 2 1.02, 3 0.97, 6 1.06, 10 0.96, 12 0.89.
+inline bool stages_alone(int links, int H, int rows, bool shared = false) {
   const bool lines = (long long)H * links % 32 == 0;
   if (links == 1 || links == 4 || links == 5 || links == 7 || links == 9) return lines && rows > 96 * device_sms();
-  return lines || (links != 11 && rows <= 192 * device_sms());
+  if (lines || links == 11 || rows > 192 * device_sms()) return lines;
+  return !shared || links == 3 || links == 8 || (links >= 10 && rows > 96 * device_sms());
 }
 
 // Dynamic shared memory of a rollout block of `block` threads staging K
@@ -91,7 +100,7 @@ __device__ __forceinline__ void chain_tip(const float (&len)[NL], const float (&
   }
 }
 
-template <int NL, int PF, int T>
+template <int NL, int PF, int T, bool SFU = kSfuTurns<NL, PF>>
 __device__ __forceinline__ void rollout_chain_body(const RolloutArgs& a, const ChainModel& cm,
                                                    int r, bool live, const StagedRows<NL, T>* st) {
   const int b = a.row0 + r;
@@ -147,7 +156,7 @@ __device__ __forceinline__ void rollout_chain_body(const RolloutArgs& a, const C
 #pragma unroll
       for (int j = 0; j < NL; ++j) {
         tau[j] = u[j];
-        sincos_reduced<kSfuTurns<NL, PF>>(phi[j], &s[j], &c[j]);
+        sincos_reduced<SFU>(phi[j], &s[j], &c[j]);
       }
       // stage cost c(x_t, u_t): reach error of the tip and torque penalty
       {
@@ -312,7 +321,7 @@ __device__ __forceinline__ void rollout_chain_body(const RolloutArgs& a, const C
     {
       float c[NL], s[NL], x, y;
 #pragma unroll
-      for (int j = 0; j < NL; ++j) sincos_reduced<kSfuTurns<NL, PF>>(phi[j], &s[j], &c[j]);
+      for (int j = 0; j < NL; ++j) sincos_reduced<SFU>(phi[j], &s[j], &c[j]);
       chain_tip<NL>(len, c, s, x, y);
       const float ex = x - cm.target[0], ey = y - cm.target[1];
       J.add(cm.w_term * cm.w_target * fmaf(ex, ex, ey * ey), a.kahan);
@@ -328,19 +337,19 @@ __device__ __forceinline__ void rollout_chain_body(const RolloutArgs& a, const C
 // Standalone launches: one thread per candidate row.  Direct loads (T = 0)
 // let threads past the last row leave at once; staged loads keep every lane
 // of a warp in the warp's copy protocol.
-template <int NL, int T>
+template <int NL, int T, bool SFU>
 __global__ void __launch_bounds__(kThreads) k_rollout_chain(const RolloutArgs a,
                                                             const ChainModel cm) {
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
   if constexpr (T == 0) {
     if (r >= a.rows) return;
-    rollout_chain_body<NL, kPrefetchAlone, 0>(a, cm, r, true, nullptr);
+    rollout_chain_body<NL, kPrefetchAlone, 0, SFU>(a, cm, r, true, nullptr);
   } else {
     if (__all_sync(0xffffffffu, r >= a.rows)) return;
     const int r0 = r & ~31;
     const StagedRows<NL, T> st{a.U + (size_t)r0 * a.H * NL, min(32, a.rows - r0),
                                warp_stage_area(StageShape<NL, T>::kWarpBytes)};
-    rollout_chain_body<NL, kPrefetchAlone, T>(a, cm, r, r < a.rows, &st);
+    rollout_chain_body<NL, kPrefetchAlone, T, SFU>(a, cm, r, r < a.rows, &st);
   }
 }
 

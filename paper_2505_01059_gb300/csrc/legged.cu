@@ -15,7 +15,8 @@
 // force at the distal end of link c acts on every phi_j with j <= c), the
 // velocity terms through the O(L) prefix / suffix form.  What a thread keeps
 // from step to step (angles, velocities, per-sample constants) lies in shared
-// memory; a step's own vectors in registers.
+// memory; a step's own vectors in registers or, where those are dearer, there too
+// (LegForm).
 #include "rollout_common.cuh"
 
 namespace mtp {
@@ -31,7 +32,32 @@ __device__ __forceinline__ float smooth_sign(float x) {
   return 1.f - __fdividef(2.f, __expf(2.f * x) + 1.f);
 }
 
+// Where a step's sines, cosines, velocity terms and suffix sums lie up to the
+// factorisation, and whether the angles' whole turns are taken by rintf on the SFU (the
+// same value).  Registers and off the SFU is the faster form (kRegisters over
+// kSharedSfu: 6 links 0.97, 13 0.93, 14 0.75 to 0.93, 16 0.95 to 1.00; 16384 candidates
+// of 16 links, 256 steps: 465 us, 491), except with 3 links (kSharedSfu; kRegisters 1.02)
+// and with 5, few candidates and shared models (1000 of 40 steps: 85.0 us, kShared 75.6,
+// kSharedSfu 88.0; others of 5 links kShared 0.93 to 1.01, kRegisters 0.95 to 1.03).  Beyond a
+// wave of warps with that many registers, two per SM sub-partition, 14 links have room for
+// a third only without (40000 candidates of 50 steps: 209 us, kSharedSfu 164), 15 lose
+// from 20000 on (24000 to 90000: 0.96 to 1.11) and 16 on short horizons (40000 of 16
+// steps: 1.02 to 1.09).
+enum class LegForm { kRegisters, kShared, kSharedSfu };
 template <int NL>
+constexpr LegForm kLegForm = NL == 3 ? LegForm::kSharedSfu : NL == 5 ? LegForm::kShared : LegForm::kRegisters;
+template <int NL>  // of many candidates
+constexpr LegForm kLegFormMany = NL == 3 || NL >= 14 ? LegForm::kSharedSfu : LegForm::kRegisters;
+template <int NL>
+bool leg_many(int rows) {
+  return rows > (NL == 15 ? 128 : 256) * device_sms();
+}
+
+// Floats of shared memory per thread.
+template <int NL, LegForm F>
+constexpr int kLegFloats = (F == LegForm::kRegisters ? 7 : 9) * NL + 2 * (NL - 1);
+
+template <int NL, LegForm F>
 __device__ __forceinline__ void rollout_legged_body(const RolloutArgs& a, const LeggedModel& lm,
                                                     int r, float* my) {
   constexpr int NC = NL - 1;   // joint torques
@@ -46,6 +72,9 @@ __device__ __forceinline__ void rollout_legged_body(const RolloutArgs& a, const 
   float* WV = my + 5 * NL * BD;
   float* SD = my + 6 * NL * BD;
   float* TN = my + 7 * NL * BD;  // torques of steps t and t + 1 (two slots of NC)
+  constexpr bool kInRegisters = F == LegForm::kRegisters;
+  float* SA = TN + 2 * NC * BD;  // not kInRegisters: velocity-term suffix sums
+  float* SB = SA + NL * BD;
 
   const int b = a.row0 + r;
   const uint32_t iter = a.d_iter ? *a.d_iter : a.iter;
@@ -111,17 +140,35 @@ __device__ __forceinline__ void rollout_legged_body(const RolloutArgs& a, const 
       float tau[NC];
 #pragma unroll
       for (int j = 0; j < NC; ++j) tau[j] = slot[j * BD];
-      // up to the factorisation a step's vectors stay in registers (the factor's
-      // own take their place); shared memory keeps the sines and cosines for the
-      // base acceleration after it
-      float c[NL], s[NL], om[NL], lb[NL];
+      // kInRegisters: up to the factorisation a step's vectors stay in registers (the
+      // factor's own take their place); shared memory keeps the sines and cosines for
+      // the base acceleration after it
+      constexpr int kKept = kInRegisters ? NL : 1;
+      float c_kept[kKept], s_kept[kKept], om_kept[kKept], lb_kept[kKept], Sa_kept[kKept], Sb_kept[kKept];
+#define MTP_LEG_VECTOR(name, memory)                       \
+  auto name = [&](int j) -> float& {                       \
+    if constexpr (kInRegisters) return name##_kept[j];     \
+    else return memory[j * BD];                            \
+  }
+      MTP_LEG_VECTOR(c, CS);
+      MTP_LEG_VECTOR(s, SN);
+      MTP_LEG_VECTOR(om, OMG);
+      MTP_LEG_VECTOR(lb, LB);
+      MTP_LEG_VECTOR(Sa, SA);  // sums over the links beyond
+      MTP_LEG_VECTOR(Sb, SB);
+#undef MTP_LEG_VECTOR
 #pragma unroll
       for (int j = 0; j < NL; ++j) {
-        sincos_reduced(PHI[j * BD], &s[j], &c[j]);
-        SN[j * BD] = s[j];
-        CS[j * BD] = c[j];
-        om[j] = OMG[j * BD];
-        lb[j] = LB[j * BD];
+        float sj, cj;
+        sincos_reduced<F == LegForm::kSharedSfu>(PHI[j * BD], &sj, &cj);
+        SN[j * BD] = sj;
+        CS[j * BD] = cj;
+        if constexpr (kInRegisters) {
+          s_kept[j] = sj;
+          c_kept[j] = cj;
+          om_kept[j] = OMG[j * BD];
+          lb_kept[j] = LB[j * BD];
+        }
       }
       // stage cost c(x_t, u_t): height, pitch and forward velocity of the
       // base link plus the torque penalty
@@ -139,18 +186,18 @@ __device__ __forceinline__ void rollout_legged_body(const RolloutArgs& a, const 
       for (int j = 0; j < NL; ++j) {
         const float tj = (j >= 1) ? tau[j - 1] : 0.f;
         const float tj1 = (j + 1 <= NC) ? tau[j] : 0.f;
-        rhs[j] = fmaf(-lm.gravity * lb[j], c[j], tj - tj1);
+        rhs[j] = fmaf(-lm.gravity * lb(j), c(j), tj - tj1);
       }
       // contact: walk from the tip back to the base, accumulating the force
       // sum over the points beyond each link
       float cx = px, cy = py, cvx = vx, cvy = vy;
 #pragma unroll
       for (int j = 0; j < NL; ++j) {
-        const float l = lm.length[j], w = om[j];
-        cx = fmaf(l, c[j], cx);
-        cy = fmaf(l, s[j], cy);
-        cvx = fmaf(-l * w, s[j], cvx);
-        cvy = fmaf(l * w, c[j], cvy);
+        const float l = lm.length[j], w = om(j);
+        cx = fmaf(l, c(j), cx);
+        cy = fmaf(l, s(j), cy);
+        cvx = fmaf(-l * w, s(j), cvx);
+        cvy = fmaf(l * w, c(j), cvy);
       }
       float Fx = 0.f, Fy = 0.f;
 #pragma unroll
@@ -163,8 +210,8 @@ __device__ __forceinline__ void rollout_legged_body(const RolloutArgs& a, const 
         Fy += fn;
         if (point >= 1) {
           const int j = point - 1;
-          const float l = lm.length[j], w = om[j];
-          const float sj = s[j], cj = c[j];
+          const float l = lm.length[j], w = om(j);
+          const float sj = s(j), cj = c(j);
           rhs[j] = fmaf(l, fmaf(-sj, Fx, cj * Fy), rhs[j]);
           cx = fmaf(-l, cj, cx);
           cy = fmaf(-l, sj, cy);
@@ -176,15 +223,14 @@ __device__ __forceinline__ void rollout_legged_body(const RolloutArgs& a, const 
       // sums), and the base equation's right-hand side
       float Rx = Fx, Ry = fmaf(-m_tot, lm.gravity, Fy);
       {
-        float Sa[NL], Sb[NL];  // sums over the links beyond
         float sum_a = 0.f, sum_b = 0.f;
 #pragma unroll
         for (int k = NL - 1; k >= 0; --k) {
-          Sa[k] = sum_a;
-          Sb[k] = sum_b;
-          const float w2 = om[k] * om[k];
-          sum_a = fmaf(lb[k], c[k] * w2, sum_a);
-          sum_b = fmaf(lb[k], s[k] * w2, sum_b);
+          Sa(k) = sum_a;
+          Sb(k) = sum_b;
+          const float w2 = om(k) * om(k);
+          sum_a = fmaf(lb(k), c(k) * w2, sum_a);
+          sum_b = fmaf(lb(k), s(k) * w2, sum_b);
         }
         Rx += sum_a;  // sum_j lb_j cos(phi_j) w_j^2
         Ry += sum_b;  // sum_j lb_j sin(phi_j) w_j^2
@@ -192,18 +238,18 @@ __device__ __forceinline__ void rollout_legged_body(const RolloutArgs& a, const 
 #pragma unroll
         for (int j = 0; j < NL; ++j) {
           const float l = lm.length[j];
-          const float ca = fmaf(lb[j], Pa, l * Sa[j]);
-          const float cb = fmaf(lb[j], Pb, l * Sb[j]);
-          rhs[j] = rhs[j] - fmaf(s[j], ca, -c[j] * cb);
-          const float w2 = om[j] * om[j];
-          Pa = fmaf(l, c[j] * w2, Pa);
-          Pb = fmaf(l, s[j] * w2, Pb);
+          const float ca = fmaf(lb(j), Pa, l * Sa(j));
+          const float cb = fmaf(lb(j), Pb, l * Sb(j));
+          rhs[j] = rhs[j] - fmaf(s(j), ca, -c(j) * cb);
+          const float w2 = om(j) * om(j);
+          Pa = fmaf(l, c(j) * w2, Pa);
+          Pb = fmaf(l, s(j) * w2, Pb);
         }
       }
       // Schur right-hand side
 #pragma unroll
       for (int j = 0; j < NL; ++j)
-        rhs[j] = fmaf(-lb[j] * invm, fmaf(-s[j], Rx, c[j] * Ry), rhs[j]);
+        rhs[j] = fmaf(-lb(j) * invm, fmaf(-s(j), Rx, c(j) * Ry), rhs[j]);
       // Schur system S phi'' = rhs.  Below the diagonal S_jk = u_j . v_k with
       // u_j = lb_j (cos phi_j, sin phi_j) and v_k = WV_k (cos phi_k, sin phi_k):
       // a rank-2 semiseparable matrix plus its diagonal SD.  Its Cholesky
@@ -217,9 +263,9 @@ __device__ __forceinline__ void rollout_legged_body(const RolloutArgs& a, const 
         float m11 = 0.f, m12 = 0.f, m22 = 0.f;
 #pragma unroll
         for (int k = 0; k < NL; ++k) {
-          const float ck = c[k], sk = s[k], wvk = WV[k * BD];
-          u1[k] = lb[k] * ck;
-          u2[k] = lb[k] * sk;
+          const float ck = c(k), sk = s(k), wvk = WV[k * BD];
+          u1[k] = lb(k) * ck;
+          u2[k] = lb(k) * sk;
           const float mu1 = fmaf(m11, u1[k], m12 * u2[k]);
           const float mu2 = fmaf(m12, u1[k], m22 * u2[k]);
           const float inv = rsqrtf(SD[k * BD] - fmaf(u1[k], mu1, u2[k] * mu2));
@@ -290,34 +336,36 @@ __device__ __forceinline__ void rollout_legged_body(const RolloutArgs& a, const 
   a.cost[r] = cst;
 }
 
-template <int NL>
+template <int NL, LegForm F>
 __global__ void __launch_bounds__(kLegThreads) k_rollout_legged(const RolloutArgs a,
                                                                 const LeggedModel lm) {
-  __shared__ float sh[(7 * NL + 2 * (NL - 1)) * kLegThreads];
+  __shared__ float sh[kLegFloats<NL, F> * kLegThreads];
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= a.rows) return;
-  rollout_legged_body<NL>(a, lm, r, sh + threadIdx.x);
+  rollout_legged_body<NL, F>(a, lm, r, sh + threadIdx.x);
 }
 
-template <int NL>
+template <int NL, LegForm F>
 __global__ void __launch_bounds__(kLegThreads) k_rollout_legged_batch(
     const RolloutArgs* __restrict__ ra, const LeggedModel* __restrict__ lms,
     const int* __restrict__ row_start, int count) {
-  __shared__ float sh[(7 * NL + 2 * (NL - 1)) * kLegThreads];
+  __shared__ float sh[kLegFloats<NL, F> * kLegThreads];
   const int g = blockIdx.x * blockDim.x + threadIdx.x;
   if (g >= __ldg(row_start + count)) return;
   const int i = batch_instance(row_start, count, g);
   const RolloutArgs a = ra[i];
   const int r = g - __ldg(row_start + i);
   if (r >= a.rows) return;
-  rollout_legged_body<NL>(a, lms[i], r, sh + threadIdx.x);
+  rollout_legged_body<NL, F>(a, lms[i], r, sh + threadIdx.x);
 }
 
 template <int NL>
 cudaError_t legged_dispatch(const RolloutArgs& a, const LeggedModel& m, int links, cudaStream_t s) {
   if constexpr (NL <= 16) {
     if (links == NL) {
-      k_rollout_legged<NL><<<(a.rows + kLegThreads - 1) / kLegThreads, kLegThreads, 0, s>>>(a, m);
+      const int blocks = (a.rows + kLegThreads - 1) / kLegThreads;
+      if (leg_many<NL>(a.rows)) k_rollout_legged<NL, kLegFormMany<NL>><<<blocks, kLegThreads, 0, s>>>(a, m);
+      else k_rollout_legged<NL, kLegForm<NL>><<<blocks, kLegThreads, 0, s>>>(a, m);
       return cudaGetLastError();
     }
     return legged_dispatch<NL + 1>(a, m, links, s);
@@ -331,8 +379,10 @@ cudaError_t legged_batch_dispatch(const RolloutArgs* ra, const LeggedModel* lm, 
                                   int count, int total_rows, int links, cudaStream_t s) {
   if constexpr (NL <= 16) {
     if (links == NL) {
-      k_rollout_legged_batch<NL><<<(total_rows + kLegThreads - 1) / kLegThreads, kLegThreads, 0, s>>>(
-          ra, lm, rs, count);
+      const int blocks = (total_rows + kLegThreads - 1) / kLegThreads;
+      if (leg_many<NL>(total_rows))
+        k_rollout_legged_batch<NL, kLegFormMany<NL>><<<blocks, kLegThreads, 0, s>>>(ra, lm, rs, count);
+      else k_rollout_legged_batch<NL, kLegForm<NL>><<<blocks, kLegThreads, 0, s>>>(ra, lm, rs, count);
       return cudaGetLastError();
     }
     return legged_batch_dispatch<NL + 1>(ra, lm, rs, count, total_rows, links, s);

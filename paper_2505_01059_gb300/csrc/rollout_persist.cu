@@ -27,7 +27,7 @@
 // CTAs per SM, i.e. at most 170 registers per thread (168 used, no spills).
 //
 // Measured on GB300 on the 256-instance batch (the bench's timed region):
-// 1.89 ms per iteration with two launches: 2.68 before the point masses
+// 1.90 ms per iteration with two launches: 2.68 before the point masses
 // evaluated several steps' costs at once (2.43 then), 2.09 before the chains'
 // controls were staged by asynchronous copies and not by bulk copies with
 // their barriers, the rest in generation.  The order of the
